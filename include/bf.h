@@ -531,7 +531,7 @@ bf_status bf_control_randomize(bf_ctx* ctx, const float* in, size_t n, uint64_t 
  *            returns once the work is enqueued; out is valid when the stream
  *            reaches it.
  * Output equals bf_control_randomize(ctx, in, n, seed, out).  The sort scratch
- * is a fixed array in the library's device code (6 MiB, held on every GPU
+ * is a fixed array in the library's device code (4.25 MiB, held on every GPU
  * that loads it until the process exits); it is shared by every call and
  * keeps the last call's contents (nothing in it needs clearing), so calls
  * whose work overlaps on the GPU, e.g. on two streams, race.

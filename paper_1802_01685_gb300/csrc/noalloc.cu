@@ -1,8 +1,8 @@
 // Time-randomised control without any device allocation.
 //
-// bf_control_randomize() takes its sort scratch (64-bit keys and 32-bit
-// indices for every sample) from the context's allocator, and it needs a
-// context, whose creation allocates too.  Some callers cannot allocate device
+// bf_control_randomize() takes its sort scratch (two 32-bit words for every
+// sample and every bucket of the sort) from the context's allocator, and it
+// needs a context, whose creation allocates too.  Some callers cannot allocate device
 // memory at the point where they need the control: code that runs inside a
 // framework whose allocator owns all device memory, pipelines that fix their
 // device-memory plan up front and must not grow it (or stall on an implicit
@@ -12,15 +12,15 @@
 // calls no cudaMalloc, cudaFree or other allocating routine.
 //
 // The array lives in the library's device code.  CUDA loads that code lazily
-// by default, so the array (BF_STATIC_CONTROL_MAX samples of scratch, 12
-// bytes per padded sample: 6 MiB) and the permutation kernels are placed in
+// by default, so the array (the scratch of BF_STATIC_CONTROL_MAX samples,
+// 4.25 MiB) and the permutation kernels are placed in
 // device memory by a set-up step: the first call on a device, or bf_init on
 // that device, loads them and looks up the array's device address.  That
 // first call may allocate through the driver; every later call allocates
 // nothing.  The array then stays until the process exits, on every GPU that
 // loaded it.  Every call shares it and finds the previous call's contents;
-// the key kernel rewrites every entry it later reads, so nothing has to start
-// at zero.  Two calls whose work overlaps on the GPU (for example on two
+// a call clears its bucket counts and rewrites every other entry it reads, so
+// nothing has to start at zero.  Two calls whose work overlaps on the GPU (for example on two
 // streams) race on the array.
 #include <mutex>
 
@@ -29,10 +29,11 @@
 
 namespace bfi {
 
-// padded sort length = next power of two >= n; keys (8 B) then indices (4 B)
+// permute_scratch_bytes of the largest call, 2^19 samples in 2^15 buckets
+// (each call checks its own need against it)
 constexpr uint64_t STATIC_CONTROL_PAD = 1ull << 19;
 static_assert(BF_STATIC_CONTROL_MAX <= STATIC_CONTROL_PAD, "scratch sized for the maximum");
-constexpr size_t STATIC_SCRATCH_BYTES = STATIC_CONTROL_PAD * (sizeof(uint64_t) + sizeof(uint32_t));
+constexpr size_t STATIC_SCRATCH_BYTES = (STATIC_CONTROL_PAD + STATIC_CONTROL_PAD / 16) * 2 * sizeof(uint32_t) + 256;
 
 static __device__ __align__(256) unsigned char g_control_scratch[STATIC_SCRATCH_BYTES];
 
@@ -108,6 +109,8 @@ extern "C" bf_status bf_control_randomize_static(const float* in, size_t n, uint
     void* scratch = nullptr;
     bf_status st = static_control_setup(dev, &scratch);
     if (st) return st;
-    e = launch_permute(in, n, seed, out, scratch, static_cast<cudaStream_t>(stream));
+    e = permute_scratch_bytes(n) <= STATIC_SCRATCH_BYTES
+            ? launch_permute(in, n, seed, out, scratch, static_cast<cudaStream_t>(stream))
+            : cudaErrorInvalidValue;
     return e == cudaSuccess ? BF_OK : cuda_fail(e, "control randomisation (static scratch)");
 }

@@ -2,15 +2,35 @@
 // with its samples permuted, which keeps the sample histogram exactly and
 // destroys all phase coherence.  The permutation is the argsort of the pairs
 // (splitmix64(seed ^ i), i) -- a counter-based draw, so it does not depend on
-// the device or thread count -- computed by a bitonic sort of 64-bit keys with
-// 32-bit indices (pads sort last), followed by a gather out[j] = in[pi(j)].
+// the device or thread count -- and out[rank of i] = in[i].
 // splitmix64 is the published generator of Steele, Lea and Flood (2014).
+//
+// The keys are as good as uniform, so one pass of buckets on their leading
+// bits leaves about 8-16 keys to a bucket (32-64 from 2^23 samples on), and a
+// key's place inside its bucket is the number of smaller pairs there:
+//   count    the bucket of every i; its slot in the bucket by arrival (atomic)
+//   scan     where each bucket begins
+//   scatter  i into its bucket, in arrival order
+//   rank     the place of i among its bucket's pairs, and the sample moved
+// Nothing is assumed of the keys but speed: any distribution gives the argsort
+// (the pairs are compared in full), a crowded bucket only takes longer, and
+// the arrival order does not reach the output.  Keys are computed again where
+// they are needed (a dozen integer operations) rather than stored, so the
+// scratch is 8 bytes a sample and 8 a bucket.  The work is latency, not
+// bandwidth: 262,144 samples on the device took 241 us a call as a bitonic sort
+// of (key, index) arrays in 37 launches, and take 42 us in these four.
+#include <algorithm>
+
 #include "bf_internal.h"
 
 namespace bfi {
 
-constexpr int SORT_CHUNK = 2048;          // elements per shared-memory block
-constexpr int SORT_THREADS = SORT_CHUNK / 2;
+constexpr int SORT_T = 256;               // threads per block of the per-sample kernels
+constexpr int SCAN_THREADS = 1024;        // of the scan; each takes four buckets
+constexpr uint32_t SCAN_TILE = 4 * SCAN_THREADS;
+constexpr uint32_t SMALL_N = 4096;        // sorted by one block, in shared memory
+constexpr int SMALL_T = 1024;
+constexpr uint32_t SMALL_BUCKETS = 1024;
 
 __device__ __forceinline__ uint64_t splitmix64(uint64_t z)
 {
@@ -20,101 +40,166 @@ __device__ __forceinline__ uint64_t splitmix64(uint64_t z)
     return z ^ (z >> 31);
 }
 
-__device__ __forceinline__ bool pair_greater(uint64_t ka, uint32_t ia, uint64_t kb, uint32_t ib)
+// (ka, ia) before (kb, ib) in the argsort's order
+__device__ __forceinline__ bool pair_less(uint64_t ka, uint32_t ia, uint64_t kb, uint32_t ib)
 {
-    return ka > kb || (ka == kb && ia > ib);
+    return ka < kb || (ka == kb && ia < ib);
 }
 
-__global__ void k_perm_keys(uint64_t* __restrict__ keys, uint32_t* __restrict__ idx, uint64_t n,
-                            uint64_t P, uint64_t seed)
+// inclusive scan over the block's threads (all of them take part); sh: one word per warp
+__device__ __forceinline__ uint32_t block_incl_scan(uint32_t v, uint32_t* sh)
 {
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < P;
-         i += (uint64_t)gridDim.x * blockDim.x) {
-        keys[i] = i < n ? splitmix64(seed ^ i) : ~0ull;
-        idx[i] = i < n ? (uint32_t)i : 0xFFFFFFFFu;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
+    uint32_t inc = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += t;
     }
-}
-
-// one compare-exchange step (k, j) over the whole array
-__global__ void k_bitonic_global(uint64_t* __restrict__ keys, uint32_t* __restrict__ idx,
-                                 uint64_t P, uint64_t j, uint64_t k)
-{
-    for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < P / 2;
-         t += (uint64_t)gridDim.x * blockDim.x) {
-        // t-th pair: i has bit j clear
-        uint64_t i = ((t & ~(j - 1)) << 1) | (t & (j - 1));
-        uint64_t l = i | j;
-        bool asc = (i & k) == 0;
-        uint64_t ka = keys[i], kb = keys[l];
-        uint32_t ia = idx[i], ib = idx[l];
-        if (pair_greater(ka, ia, kb, ib) == asc) {
-            keys[i] = kb; keys[l] = ka;
-            idx[i] = ib; idx[l] = ia;
+    if (lane == 31) sh[wid] = inc;
+    __syncthreads();
+    if (wid == 0) {
+        uint32_t s = lane < nw ? sh[lane] : 0u;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, s, o);
+            if (lane >= o) s += t;
         }
-    }
-}
-
-// all steps with j < chunk for stages k in [k_lo, k_hi], in shared memory;
-// the first stage starts at j_start
-__global__ void __launch_bounds__(SORT_THREADS) k_bitonic_shared(uint64_t* __restrict__ keys,
-                                                                 uint32_t* __restrict__ idx,
-                                                                 uint64_t chunk, uint64_t k_lo,
-                                                                 uint64_t k_hi, uint64_t j_start)
-{
-    __shared__ uint64_t sk[SORT_CHUNK];
-    __shared__ uint32_t si[SORT_CHUNK];
-    const uint64_t base = (uint64_t)blockIdx.x * chunk;
-    for (uint64_t e = threadIdx.x; e < chunk; e += blockDim.x) {
-        sk[e] = keys[base + e];
-        si[e] = idx[base + e];
+        if (lane < nw) sh[lane] = s;
     }
     __syncthreads();
-    for (uint64_t k = k_lo; k <= k_hi; k <<= 1) {
-        for (uint64_t j = (k == k_lo ? j_start : k >> 1); j > 0; j >>= 1) {
-            for (uint64_t t = threadIdx.x; t < chunk / 2; t += blockDim.x) {
-                uint64_t i = ((t & ~(j - 1)) << 1) | (t & (j - 1));
-                uint64_t l = i | j;
-                bool asc = ((base + i) & k) == 0;
-                if (pair_greater(sk[i], si[i], sk[l], si[l]) == asc) {
-                    uint64_t tk = sk[i]; sk[i] = sk[l]; sk[l] = tk;
-                    uint32_t ti = si[i]; si[i] = si[l]; si[l] = ti;
-                }
-            }
-            __syncthreads();
+    return inc + (wid > 0 ? sh[wid - 1] : 0u);
+}
+
+// count[b] (zeroed before) and slot[i], bucket b = the key's bits above `shift`
+__global__ void __launch_bounds__(SORT_T) k_perm_count(uint32_t n, uint64_t seed, int shift,
+                                                       uint32_t* __restrict__ count, uint32_t* __restrict__ slot)
+{
+    const uint64_t i = blockIdx.x * (uint64_t)SORT_T + threadIdx.x;
+    if (i >= n) return;
+    slot[i] = atomicAdd(count + (splitmix64(seed ^ i) >> shift), 1u);
+}
+
+// begin[b] = the samples in buckets before b.  Every block scans its own
+// SCAN_TILE buckets and sums all those before them itself, so that no block
+// waits for another and one launch does (the last of 8 tiles at 2^19 samples
+// reads 112 KB from L2).  n_buckets is a multiple of 4.
+__global__ void __launch_bounds__(SCAN_THREADS) k_perm_scan(const uint32_t* __restrict__ count, uint32_t n_buckets,
+                                                            uint32_t* __restrict__ begin)
+{
+    __shared__ uint32_t sh[SCAN_THREADS / 32];
+    __shared__ uint32_t sh_base;
+    const uint4* c4 = reinterpret_cast<const uint4*>(count);
+    const uint32_t q = blockIdx.x * SCAN_THREADS + threadIdx.x;        // this thread's four buckets
+    uint32_t before = 0;
+    for (uint32_t p = threadIdx.x; p < blockIdx.x * SCAN_THREADS; p += SCAN_THREADS) {
+        const uint4 v = c4[p];
+        before += (v.x + v.y) + (v.z + v.w);
+    }
+    const uint32_t all = block_incl_scan(before, sh);
+    if (threadIdx.x == SCAN_THREADS - 1) sh_base = all;
+    __syncthreads();
+    const uint32_t base = sh_base;
+    const bool in = 4 * q < n_buckets;
+    const uint4 v = in ? c4[q] : make_uint4(0u, 0u, 0u, 0u);
+    const uint32_t mine = (v.x + v.y) + (v.z + v.w);
+    const uint32_t e = base + block_incl_scan(mine, sh) - mine;
+    if (in) reinterpret_cast<uint4*>(begin)[q] = make_uint4(e, e + v.x, e + v.x + v.y, e + v.x + v.y + v.z);
+}
+
+__global__ void __launch_bounds__(SORT_T) k_perm_scatter(uint32_t n, uint64_t seed, int shift,
+                                                         const uint32_t* __restrict__ begin,
+                                                         const uint32_t* __restrict__ slot,
+                                                         uint32_t* __restrict__ idx)
+{
+    const uint64_t i = blockIdx.x * (uint64_t)SORT_T + threadIdx.x;
+    if (i >= n) return;
+    idx[begin[splitmix64(seed ^ i) >> shift] + slot[i]] = (uint32_t)i;
+}
+
+// One thread per place p of the bucket order: its sample's final place is its
+// bucket's beginning plus the number of smaller pairs in the bucket.
+__global__ void __launch_bounds__(SORT_T) k_perm_rank(const float* __restrict__ in, uint32_t n, uint64_t seed,
+                                                      int shift, const uint32_t* __restrict__ begin,
+                                                      const uint32_t* __restrict__ count,
+                                                      const uint32_t* __restrict__ idx, float* __restrict__ out)
+{
+    const uint64_t p = blockIdx.x * (uint64_t)SORT_T + threadIdx.x;
+    if (p >= n) return;
+    const uint32_t i = idx[p];
+    const float v = in[i];
+    const uint64_t key = splitmix64(seed ^ (uint64_t)i);
+    const uint32_t b0 = begin[key >> shift], m = count[key >> shift];
+    uint32_t rank = b0;
+#pragma unroll 4
+    for (uint32_t q = 0; q < m; ++q) {
+        const uint32_t j = idx[b0 + q];
+        rank += pair_less(splitmix64(seed ^ (uint64_t)j), j, key, i) ? 1u : 0u;
+    }
+    out[rank] = v;
+}
+
+// The four steps in one block for n <= SMALL_N.
+__global__ void __launch_bounds__(SMALL_T) k_perm_small(const float* __restrict__ in, uint32_t n, uint64_t seed,
+                                                        float* __restrict__ out)
+{
+    __shared__ uint32_t count[SMALL_BUCKETS], begin[SMALL_BUCKETS];
+    __shared__ uint32_t sh[SMALL_T / 32];
+    __shared__ uint64_t key[SMALL_N];
+    __shared__ uint32_t idx[SMALL_N];
+    constexpr int E = SMALL_N / SMALL_T;
+    constexpr int SHIFT = 54;                                  // 2^10 buckets
+    static_assert(SMALL_BUCKETS == 1024 && SMALL_T == 1024, "one thread per bucket");
+    count[threadIdx.x] = 0u;
+    __syncthreads();
+    uint64_t k[E];
+    uint32_t slot[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const uint32_t i = threadIdx.x + e * SMALL_T;
+        k[e] = splitmix64(seed ^ (uint64_t)i);
+        if (i < n) slot[e] = atomicAdd(count + (k[e] >> SHIFT), 1u);
+    }
+    __syncthreads();
+    const uint32_t c = count[threadIdx.x];
+    begin[threadIdx.x] = block_incl_scan(c, sh) - c;
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const uint32_t i = threadIdx.x + e * SMALL_T;
+        if (i < n) {
+            const uint32_t p = begin[k[e] >> SHIFT] + slot[e];
+            key[p] = k[e];
+            idx[p] = i;
         }
     }
-    for (uint64_t e = threadIdx.x; e < chunk; e += blockDim.x) {
-        keys[base + e] = sk[e];
-        idx[base + e] = si[e];
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const uint32_t i = threadIdx.x + e * SMALL_T;
+        if (i >= n) continue;
+        const uint32_t b0 = begin[k[e] >> SHIFT], m = count[k[e] >> SHIFT];
+        uint32_t rank = b0;
+        for (uint32_t q = b0; q < b0 + m; ++q) rank += pair_less(key[q], idx[q], k[e], i) ? 1u : 0u;
+        out[rank] = in[i];
     }
 }
 
-__global__ void k_gather(const float* __restrict__ in, const uint32_t* __restrict__ idx,
-                         uint64_t n, float* __restrict__ out)
+// log2 of the number of buckets for n > SMALL_N samples: 8-16 samples a bucket
+// up to 2^23 samples (2^19 buckets), where the scan's re-reading of the tiles
+// before each block is still microseconds; 32-64 beyond
+static int bucket_bits(uint64_t n)
 {
-    for (uint64_t j = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; j < n;
-         j += (uint64_t)gridDim.x * blockDim.x)
-        out[j] = in[idx[j]];
-}
-
-static uint64_t pow2_at_least(uint64_t n)
-{
-    uint64_t P = 1;
-    while (P < n) P <<= 1;
-    return P < 2 ? 2 : P;
+    int p = 0;
+    while ((1ull << p) < n) ++p;           // 2^p >= n
+    return n <= (1ull << 23) ? p - 4 : p - 6;
 }
 
 size_t permute_scratch_bytes(uint64_t n)
 {
-    uint64_t P = pow2_at_least(n);
-    return (size_t)P * (sizeof(uint64_t) + sizeof(uint32_t)) + 256;
-}
-
-static unsigned grid_for(uint64_t work)
-{
-    uint64_t b = (work + 255) / 256;
-    if (b > 65535ull * 16) b = 65535ull * 16;
-    return (unsigned)(b ? b : 1);
+    if (n <= SMALL_N) return 256;
+    const uint64_t B = 1ull << bucket_bits(n);
+    return (size_t)((B + n) * 2 * sizeof(uint32_t)) + 256;
 }
 
 // Loads the code of the permutation kernels on the current device.  Under
@@ -124,36 +209,39 @@ static unsigned grid_for(uint64_t work)
 cudaError_t preload_permute()
 {
     cudaFuncAttributes a;
-    cudaError_t e = cudaFuncGetAttributes(&a, k_perm_keys);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_bitonic_shared);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_bitonic_global);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_gather);
+    cudaError_t e = cudaFuncGetAttributes(&a, k_perm_count);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_perm_scan);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_perm_scatter);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_perm_rank);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_perm_small);
     return e;
 }
 
+// n < 2^32 - 1 (the callers check)
 cudaError_t launch_permute(const float* in, uint64_t n, uint64_t seed, float* out, void* scratch,
                            cudaStream_t s)
 {
     if (n == 0) return cudaSuccess;
-    const uint64_t P = pow2_at_least(n);
-    uint64_t* keys = reinterpret_cast<uint64_t*>(scratch);
-    uint32_t* idx = reinterpret_cast<uint32_t*>(keys + P);
-    count_launches(1);
-    k_perm_keys<<<grid_for(P), 256, 0, s>>>(keys, idx, n, P, seed);
-    const uint64_t chunk = P < (uint64_t)SORT_CHUNK ? P : (uint64_t)SORT_CHUNK;
-    const unsigned nchunks = (unsigned)(P / chunk);
-    count_launches(1);
-    k_bitonic_shared<<<nchunks, SORT_THREADS, 0, s>>>(keys, idx, chunk, 2, chunk, 1);
-    for (uint64_t k = chunk << 1; k <= P; k <<= 1) {
-        for (uint64_t j = k >> 1; j >= chunk; j >>= 1) {
-            count_launches(1);
-            k_bitonic_global<<<grid_for(P / 2), 256, 0, s>>>(keys, idx, P, j, k);
-        }
+    if (n > 0xFFFFFFFFull) return cudaErrorInvalidValue;
+    if (n <= SMALL_N) {
         count_launches(1);
-        k_bitonic_shared<<<nchunks, SORT_THREADS, 0, s>>>(keys, idx, chunk, k, k, chunk >> 1);
+        k_perm_small<<<1, SMALL_T, 0, s>>>(in, (uint32_t)n, seed, out);
+        return cudaGetLastError();
     }
-    count_launches(1);
-    k_gather<<<grid_for(n), 256, 0, s>>>(in, idx, n, out);
+    const int bits = bucket_bits(n), shift = 64 - bits;
+    const uint32_t B = 1u << bits;
+    uint32_t* count = reinterpret_cast<uint32_t*>(scratch);        // [B], 16-byte aligned
+    uint32_t* begin = count + B;
+    uint32_t* slot = begin + B;
+    uint32_t* idx = slot + n;
+    cudaError_t e = cudaMemsetAsync(count, 0, (size_t)B * sizeof(uint32_t), s);
+    if (e != cudaSuccess) return e;
+    const unsigned grid = (unsigned)((n + SORT_T - 1) / SORT_T);
+    count_launches(4);
+    k_perm_count<<<grid, SORT_T, 0, s>>>((uint32_t)n, seed, shift, count, slot);
+    k_perm_scan<<<(B + SCAN_TILE - 1) / SCAN_TILE, SCAN_THREADS, 0, s>>>(count, B, begin);
+    k_perm_scatter<<<grid, SORT_T, 0, s>>>((uint32_t)n, seed, shift, begin, slot, idx);
+    k_perm_rank<<<grid, SORT_T, 0, s>>>(in, (uint32_t)n, seed, shift, begin, count, idx, out);
     return cudaGetLastError();
 }
 
