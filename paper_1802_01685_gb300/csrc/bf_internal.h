@@ -329,7 +329,7 @@ cudaError_t launch_template_power_dot(const float* rows, uint32_t n_rows, const 
 uint32_t fft_seg_len(bool quad);            // samples per segment
 uint32_t fft_spec_bins(bool quad);          // complex bins per segment or template spectrum
 uint32_t fft_lags_per_seg(uint32_t M, bool quad);          // V = fft_seg_len - M + 1
-uint32_t fft_norm_stride(uint32_t M, bool quad);           // Vp: V rounded up to a multiple of 4
+uint32_t fft_norm_stride(uint32_t M, bool quad);           // Vp: V rounded up to whole rounds of outputs
 float fft_inverse_scale(bool quad);
 // a series' FFT-route scratch: its segment spectra [nseg][fft_spec_bins],
 // then its window norms per segment [nseg][fft_norm_stride] (fft_seg_norms)

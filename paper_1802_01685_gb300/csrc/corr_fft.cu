@@ -31,31 +31,20 @@
 //  * template spectra are kept by a stored bank in HBM (made once) and made
 //    per call for a generated bank, chunk by chunk, in a two-slot ring on the
 //    auxiliary stream;
-//  * each segment spectrum is computed once per call; all of them stay in L2
-//    and reach shared memory by asynchronous copies (cp.async) issued one
-//    segment ahead; the segment's window norms are read from L2 straight
-//    into registers;
-//  * one CTA of 512 threads owns a template (real route) or a pair (pair
-//    route) at a time and holds its spectra in registers (16 bins per
-//    thread).  For every segment it forms the product spectrum; the first FFT
-//    pass reads, per thread, 8 bins it formed itself and 8 that the mirror
-//    thread formed (Hermitian symmetry), exchanged through shared memory; it
-//    runs one inverse transform in shared memory, alternating between two
-//    work arrays, and reduces the output in registers, with a warp-level
-//    test before the max/argmax and tail work.  The last radix-2 stage of the
-//    FFT is fused into the epilogue, so the filter output never reaches HBM.
-//  * The FFT is a Stockham autosort FFT with three radix-16 passes (each
-//    thread one 16-point DFT per pass, in registers) and a final radix-2
-//    stage; the work array holds complex values with index i stored at
-//    i + i/16, so that every pass moves a warp's 64-bit values in the
-//    minimum two wavefronts, and every thread addresses it at fixed offsets
-//    from one base.  Twiddles: the second pass reads a [15][16] table, the
-//    third reads e^{2 pi i r k / 4096} for r = 1, 2, 3, 4, 8, 12 and forms the
-//    others as one product of two; the last stage and the real route's
-//    even/odd split use per-thread constants e^{i pi tid / 4096} and
-//    e^{i pi tid / 8192} (rounded from FP64 once per thread) times exact-
-//    to-rounding roots of unity.  The tables are rounded from FP64 once per
-//    context and copied into shared memory by every CTA.
+//  * each segment spectrum is computed once per call; all of them stay in L2,
+//    and so do the segments' window norms, and go straight into registers;
+//  * the forward transforms (segments, templates, the predictor) are Stockham
+//    autosort FFTs of one CTA with three radix-16 passes (each thread one
+//    16-point DFT per pass, in registers) and a final radix-2 stage; the work
+//    array holds index i at i + i/16, so that every pass moves a warp's 64-bit
+//    values in the minimum two wavefronts.  Twiddles: the second pass reads a
+//    [15][16] table, the third reads e^{2 pi i r k / 4096} for r = 1, 2, 3, 4, 8, 12
+//    and forms the others as one product of two; the last stage and the real
+//    route's even/odd split use per-thread constants (rounded from FP64 once
+//    per thread) times exact-to-rounding roots of unity;
+//  * the inverse transforms, nearly all of the work, are k_corr_fft's: the
+//    product with a template's spectrum, the transform and the reduction of its
+//    output in one kernel, so that the filter output never reaches HBM.
 //  * The transform's rounding error scales with its whole segment, so lags
 //    whose window holds almost none of the segment's energy are taken out of
 //    the FFT route (k_fft_flags) and computed directly (k_fft_fixup).
@@ -78,17 +67,43 @@ constexpr int UPPER = FH + FH / 16;       // padded distance of elements 4096 ap
 // twiddle tables e^{+2 pi i n / 8192}: pass 2 [15][16] (r (j mod 16) units of
 // 32), pass 3 [6][256] (r (j mod 256) units of 2 for r = 1, 2, 3, 4, 8, 12)
 constexpr int TW2 = 0, TW3 = 15 * 16, TW_N = TW3 + 6 * 256;     // 1776 entries
-// shared memory: work array, twiddles, then (correlation only) a second work
-// array, so that the passes alternate between the two, and the staged segment
-// spectrum (FH bins on the pair route, FN on the real route)
+// shared memory of the forward transforms: work array, twiddles, then (template
+// spectra of the real route only) a second work array, so that the passes
+// alternate between the two, and the staged row
 constexpr size_t FFT_SMEM = (ZPAD + TW_N) * sizeof(float2);
-constexpr size_t CORR_SMEM = FFT_SMEM + ZPAD * sizeof(float2) + FH * sizeof(float2);
-constexpr size_t RCORR_SMEM = FFT_SMEM + ZPAD * sizeof(float2) + FN * sizeof(float2);
-static_assert(RCORR_SMEM <= 227 * 1024, "real-route correlation fits one SM's shared memory");
+constexpr size_t BANK_SMEM = FFT_SMEM + ZPAD * sizeof(float2) + FH * sizeof(float2);
 static_assert(FFT_SMEM % 16 == 0 && (FFT_SMEM + ZPAD * sizeof(float2)) % 16 == 0, "16-byte staging");
+// the correlation kernel: two groups of GT threads, each with a work array of
+// 16 blocks of 16 rows of 16 packed values at a pitch of 17 (so that the last
+// pass, whose threads differ in the row, meets no bank conflict), a template's
+// records, and twiddles: [6][256] of pass 1, e^{2 pi i q j / 4096} for q = 1, 2,
+// 3, 4, 8, 12, [15][16] of pass 2, e^{2 pi i q n / 256}, and [256][2] of the
+// product, e^{i pi j / 8192} and e^{i pi j / 4096}
+constexpr int GT = FT / 2;
+constexpr int ZROW = 17, ZBLK = 16 * ZROW, ZG = 16 * ZBLK;
+constexpr int TWC_N = 6 * 256 + 15 * 16 + 2 * 256;          // float2 entries, after the TW_N of the forward transforms
+constexpr size_t CORR_SMEM = (size_t)(2 * ZG + FH + TWC_N / 2 + 2 * 9 + FT / 32) * sizeof(float4);   // 2 x 9: column 0; the warps' reductions
+static_assert(CORR_SMEM <= 227 * 1024, "the correlation kernel fits one SM's shared memory");
+static_assert(TW_N % 2 == 0 && TWC_N % 2 == 0, "16-byte tables");
 
 __global__ void k_fft_tables(float2* __restrict__ tw)
 {
+    // the correlation kernel's tables
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < TWC_N; e += gridDim.x * blockDim.x) {
+        double a;                                 // the angle over pi
+        if (e < 6 * 256) {
+            const int q = e / 256;
+            a = (double)((q < 3 ? q + 1 : 4 * (q - 2)) * (e % 256)) / 2048.0;
+        } else if (e < 6 * 256 + 15 * 16) {
+            a = (double)(((e - 6 * 256) / 16 + 1) * (e % 16)) / 128.0;
+        } else {
+            const int i = e - 6 * 256 - 15 * 16;
+            a = (double)(i / 2) / (i % 2 ? 4096.0 : 8192.0);
+        }
+        double sn, cs;
+        sincospi(a, &sn, &cs);
+        tw[TW_N + e] = make_float2((float)cs, (float)sn);
+    }
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < TW_N; e += gridDim.x * blockDim.x) {
         int n;                                    // exponent in units of 2 pi / 8192
         if (e < TW3) {
@@ -373,17 +388,69 @@ __device__ __forceinline__ void real_spectrum(const Smem& m, float2 base_f, floa
     }
 }
 
-// the spectrum as out[0 .. N), out[0] = (S[0], S[N])
-__device__ __forceinline__ void real_spectrum_out(const Smem& m, float2 base_f, float2 base_r,
-                                                  float2* __restrict__ out)
+// U[n], U[n + 4096], U[4096 - n], U[8192 - n] of the complex transform in the
+// work array after fft_passes<-1>, n = tid + 512 i, i < 4; for n = 0 the last two
+// are U[2048] and U[6144]
+__device__ __forceinline__ void quad_bins(const float2* z, float2 base_f, int i, float2 (&u)[4])
 {
-    real_spectrum(m, base_f, base_r, [&](int, int, int k, float2 v) { out[k] = v; });
+    const int n = threadIdx.x + FT * i;
+    const float2 w = final_tw<-1>(base_f, i);
+    fft_final(z, i, w, u[0], u[1]);
+    const int m = n ? FH - n : FH / 2;
+    const int a = m + (m >> 4);
+    const float2 v = z[a + UPPER], c = z[a];
+    float vr = v.x, vi = v.y;
+    rotate(vr, vi, n ? make_float2(-w.x, w.y) : make_float2(0.f, -1.f));    // e^{-i pi m / 4096}
+    u[2] = make_float2(c.x + vr, c.y + vi);
+    u[3] = make_float2(c.x - vr, c.y - vi);
 }
 
-// Spectra of segments of a batch of series.  Pair route (F = 8192): the real
-// segment through one complex transform, half spectrum of 4096 bins with bin
-// 0 = (DC, Nyquist).  Real route (F = 16384): even/odd packed, 8192 bins with
-// bin 0 = (DC, Nyquist).
+__device__ __forceinline__ float4 lanes(float2 a, float2 b) { return make_float4(a.x, b.x, a.y, b.y); }
+
+// S[k] and S[N - k] from U[k] and U[N - k], w = e^{i pi k / N} (real_spectrum)
+__device__ __forceinline__ void real_split(float2 uk, float2 um, float2 w, float2& sk, float2& sm)
+{
+    const float2 e = make_float2(0.5f * (uk.x + um.x), 0.5f * (uk.y - um.y));
+    const float2 o = make_float2(0.5f * (uk.y + um.y), -0.5f * (uk.x - um.x));
+    const float2 wo = cmul(make_float2(w.x, -w.y), o);
+    sk = make_float2(e.x + wo.x, e.y + wo.y);
+    sm = make_float2(e.x - wo.x, wo.y - e.y);
+}
+
+// The half spectrum of a real signal (as real_spectrum) as the records the
+// correlation kernel reads: for n = j + 256 r < 2048, float4 number 2 r 256 + j
+// holds the bins n and 4096 - n as (re, re, im, im), number (2 r + 1) 256 + j the
+// bins 8192 - n and 4096 + n; the record of n = 0 holds bin 0 = (S[0], S[N]), bin
+// 4096, bin 6144 and bin 2048.
+__device__ __forceinline__ void real_spectrum_quads(const Smem& m, float2 base_f, float2 base_r,
+                                                    float2* __restrict__ out)
+{
+    const int tid = threadIdx.x;
+    float4* rec = reinterpret_cast<float4*>(out) + 2 * GT * (tid / GT) + tid % GT;
+#pragma unroll
+    for (int i = 0; i < FBINS / 2; ++i) {
+        float2 u[4], s0, s1, s2, s3;                  // bins n, 4096 - n, 8192 - n, 4096 + n
+        quad_bins(m.z, base_f, i, u);
+        if (tid == 0 && i == 0) {
+            s0 = make_float2(u[0].x + u[0].y, u[0].x - u[0].y);
+            s1 = make_float2(u[1].x, -u[1].y);
+            constexpr float R2 = 0.707106781186547524f;
+            real_split(u[2], u[3], make_float2(R2, R2), s3, s2);
+        } else {
+            const float2 w = cmul(base_r, root32(i));                        // e^{i pi n / N}
+            real_split(u[0], u[3], w, s0, s2);
+            real_split(u[2], u[1], make_float2(w.y, w.x), s1, s3);           // e^{i pi (4096 - n) / N}
+        }
+        rec[4 * GT * i] = lanes(s0, s1);
+        rec[4 * GT * i + GT] = lanes(s2, s3);
+    }
+}
+
+// Spectra of segments of a batch of series, as the correlation kernel's
+// records.  Pair route (F = 8192): the real segment through one complex
+// transform, 4096 bins: for n = j + 256 r < 2048, float4 number r 256 + j holds
+// the bins n and 4096 - n (for n = 0: bin 0 = (DC, Nyquist) and bin 2048).  Real
+// route (F = 16384): even/odd packed, 8192 bins (real_spectrum_quads).
 template <bool REAL>
 __global__ void __launch_bounds__(FT, 1) k_fft_series(const __grid_constant__ FftSeriesBatch p,
                                                       uint32_t total)
@@ -409,14 +476,14 @@ __global__ void __launch_bounds__(FT, 1) k_fft_series(const __grid_constant__ Ff
         __syncthreads();
         fft_passes<-1>(m);
         if (REAL) {
-            real_spectrum_out(m, base_f, base_r, p.spec[s] + (size_t)j * FN);
+            real_spectrum_quads(m, base_f, base_r, p.spec[s] + (size_t)j * FN);
         } else {
-            float2* out = p.spec[s] + (size_t)j * FH;
+            float4* rec = reinterpret_cast<float4*>(p.spec[s] + (size_t)j * FH) + tid;
 #pragma unroll
-            for (int i = 0; i < FBINS; ++i) {
-                float2 lo, hi;
-                fft_final(m.z, i, final_tw<-1>(base_f, i), lo, hi);
-                out[tid + FT * i] = (tid == 0 && i == 0) ? make_float2(lo.x, hi.x) : lo;
+            for (int i = 0; i < FBINS / 2; ++i) {
+                float2 u[4];
+                quad_bins(m.z, base_f, i, u);
+                rec[FT * i] = lanes(tid == 0 && i == 0 ? make_float2(u[0].x, u[1].x) : u[0], u[2]);
             }
         }
         __syncthreads();
@@ -426,7 +493,7 @@ __global__ void __launch_bounds__(FT, 1) k_fft_series(const __grid_constant__ Ff
 // Template spectra of a chunk of synthesised rows (rows of 8192 samples, zero
 // past M), pair route: rows (2q, 2q + 1) through one complex transform of
 // h_a + i h_b, separated by Hermitian symmetry into two half spectra of 4096
-// bins.
+// bins (records as k_fft_series' pair route).
 __global__ void __launch_bounds__(FT, 1) k_fft_bank_pair(const float* __restrict__ rows, uint32_t n_rows,
                                                          uint32_t n_items, const float2* __restrict__ tw,
                                                          float2* __restrict__ spec)
@@ -441,23 +508,22 @@ __global__ void __launch_bounds__(FT, 1) k_fft_bank_pair(const float* __restrict
         for (int n = tid; n < FN; n += FT) m.z[n + (n >> 4)] = make_float2(ra[n], b < n_rows ? rb[n] : 0.f);
         __syncthreads();
         fft_passes<-1>(m);
-        float2* sa = spec + (size_t)a * FH;
-        float2* sb = spec + (size_t)b * FH;
+        float4* sa = reinterpret_cast<float4*>(spec + (size_t)a * FH) + tid;
+        float4* sb = reinterpret_cast<float4*>(spec + (size_t)b * FH) + tid;
 #pragma unroll
-        for (int i = 0; i < FBINS; ++i) {
-            const int k = tid + FT * i;
-            const float2 w = final_tw<-1>(base_f, i);
-            float2 zk, zn;
-            fft_final(m.z, i, w, zk, zn);          // Z[k], Z[k + 4096]
-            if (k == 0) {
-                // DC and Nyquist of both real templates: real parts of Z[0], Z[4096]
-                sa[0] = make_float2(zk.x, zn.x);
-                if (b < n_rows) sb[0] = make_float2(zk.y, zn.y);
+        for (int i = 0; i < FBINS / 2; ++i) {
+            float2 u[4];                           // Z[n], Z[n + 4096], Z[4096 - n], Z[8192 - n]
+            quad_bins(m.z, base_f, i, u);
+            // H_a = (Z[k] + conj Z[F-k]) / 2,  H_b = (Z[k] - conj Z[F-k]) / 2i
+            auto ha = [](float2 k, float2 c) { return make_float2(0.5f * (k.x + c.x), 0.5f * (k.y - c.y)); };
+            auto hb = [](float2 k, float2 c) { return make_float2(0.5f * (k.y + c.y), -0.5f * (k.x - c.x)); };
+            if (tid == 0 && i == 0) {
+                // DC and Nyquist of both real templates: real parts of Z[0], Z[4096]; bin 2048
+                sa[0] = lanes(make_float2(u[0].x, u[1].x), ha(u[2], u[3]));
+                if (b < n_rows) sb[0] = lanes(make_float2(u[0].y, u[1].y), hb(u[2], u[3]));
             } else {
-                const float2 zm = fft_final_mirror(m.z, k, w);    // Z[F - k]
-                // H_a = (Z[k] + conj Z[F-k]) / 2,  H_b = (Z[k] - conj Z[F-k]) / 2i
-                sa[k] = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
-                if (b < n_rows) sb[k] = make_float2(0.5f * (zk.y + zm.y), -0.5f * (zk.x - zm.x));
+                sa[FT * i] = lanes(ha(u[0], u[3]), ha(u[2], u[1]));
+                if (b < n_rows) sb[FT * i] = lanes(hb(u[0], u[3]), hb(u[2], u[1]));
             }
         }
         __syncthreads();
@@ -507,7 +573,7 @@ __global__ void __launch_bounds__(FT, 1) k_fft_bank_real(const float* __restrict
         cp_async_commit();
         pass16<-1, 16, -1, false>(m, m.z, m.z2);
         pass16<-1, 256, -1, false>(m, m.z2, m.z);
-        real_spectrum_out(m, base_f, base_r, spec + (size_t)q * FN);
+        real_spectrum_quads(m, base_f, base_r, spec + (size_t)q * FN);
         if (qn >= n_rows) break;
         q = qn;
     }
@@ -640,35 +706,10 @@ __device__ __forceinline__ void push_tail(const FftParams& p, uint32_t series, u
     if (i < p.cand_cap) p.cand[i] = Candidate{series, k, tau, rho};
 }
 
-// running max |rho| with its first lag, as the packed key of pack_max (|rho|
-// >= 0, so its bits order as its values; then the lower lag): one unsigned
-// 64-bit max per update, whatever order the lags arrive in
-__device__ __forceinline__ void track_max(float a, uint32_t tau, unsigned long long& best)
-{
-    const unsigned long long key = pack_max(a, tau);
-    best = key > best ? key : best;
-}
-
-// the largest of the warp's packed keys: the largest value bits, then among
-// the lanes that hold them the largest low word (the earliest lag)
-__device__ __forceinline__ unsigned long long warp_max_key(unsigned long long k)
-{
-    const uint32_t hi = __reduce_max_sync(0xffffffffu, (uint32_t)(k >> 32));
-    const uint32_t lo = __reduce_max_sync(0xffffffffu, (uint32_t)(k >> 32) == hi ? (uint32_t)k : 0u);
-    return ((unsigned long long)hi << 32) | lo;
-}
-
 // the warp's largest of the non-negative g (float bits order as values)
 __device__ __forceinline__ float warp_max_abs(float g)
 {
     return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(g)));
-}
-
-// segment spectrum of NX bins into shared memory (16-byte asynchronous copies)
-template <int NX>
-__device__ __forceinline__ void stage_spectrum(const Smem& m, const float2* src)
-{
-    for (int c = threadIdx.x; c < NX / 2; c += FT) cp_async16(m.x + 2 * c, src + 2 * c);
 }
 
 // a 128-byte line from DRAM into L2 (no register, no wait)
@@ -677,407 +718,494 @@ __device__ __forceinline__ void prefetch_l2(const void* g)
     asm volatile("prefetch.global.L2 [%0];\n" ::"l"(g));
 }
 
-// warp reduction of a packed max key and a sum, then one atomic each per warp
-__device__ __forceinline__ void publish(unsigned long long key, double d, unsigned long long* vmax,
-                                       double* sumsq)
+// ---- The correlation kernel's transform: N = 8192 points by a group of 256
+// threads, packed two to a register pair (Blackwell's FFMA2/FADD2/FMUL2 take
+// two FP32 values per lane at half the issue rate and the full flop rate).
+// The first radix-2 stage is taken while the product spectrum is formed:
+//   a[n] = Z[n] + Z[n + 4096],  b[n] = (Z[n] - Z[n + 4096]) e^{2 pi i n / 8192},
+// n < 4096, give the outputs 2k and 2k + 1 as two 4096-point transforms, which
+// run side by side in the two halves of every register pair with the same
+// twiddles.  Each is 16 x 16 x 16, decimated in frequency and in place: with
+// n = 256 n2 + 16 n1 + n0, pass 1 turns n2 into k0, pass 2 n1 into k1, pass 3
+// n0 into k2, k = k0 + 16 k1 + 256 k2, every thread writing back to the slots
+// it read, so one array serves.  Passes 2 and 3 of a block of equal k0 belong to
+// one half-warp: only pass 1 crosses warps, so a group meets at two barriers a
+// transform (before and after pass 1 writes) and its warps drift apart between
+// them, some in shared memory while others compute.
+
+// two complex values, one per register half
+struct cpk {
+    float2 r, i;
+};
+
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, neg2(b)); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+
+// v *= (wr + i wi), lane by lane
+__device__ __forceinline__ void rotate2(cpk& v, float2 wr, float2 wi)
+{
+    const float2 r = fma2(v.r, wr, neg2(mul2(v.i, wi)));
+    v.i = fma2(v.r, wi, mul2(v.i, wr));
+    v.r = r;
+}
+
+// dft4<+1> and dft16<+1> on packed values
+__device__ __forceinline__ void dft4_pk(cpk& a, cpk& b, cpk& c, cpk& d)
+{
+    const cpk t0{add2(a.r, c.r), add2(a.i, c.i)}, t1{sub2(a.r, c.r), sub2(a.i, c.i)};
+    const cpk t2{add2(b.r, d.r), add2(b.i, d.i)}, t3{sub2(b.r, d.r), sub2(b.i, d.i)};
+    a = {add2(t0.r, t2.r), add2(t0.i, t2.i)};
+    c = {sub2(t0.r, t2.r), sub2(t0.i, t2.i)};
+    b = {sub2(t1.r, t3.i), add2(t1.i, t3.r)};
+    d = {add2(t1.r, t3.i), sub2(t1.i, t3.r)};
+}
+
+__device__ __forceinline__ void dft16_pk(cpk (&v)[16])
 {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long ok = __shfl_xor_sync(0xffffffffu, key, o);
-        key = ok > key ? ok : key;
-        d += __shfl_xor_sync(0xffffffffu, d, o);
+    for (int n2 = 0; n2 < 4; ++n2) dft4_pk(v[n2], v[4 + n2], v[8 + n2], v[12 + n2]);
+    constexpr float C1 = 0.923879532511286756f;   // cos(pi/8)
+    constexpr float S1 = 0.382683432365089772f;   // sin(pi/8)
+    constexpr float R2 = 0.707106781186547524f;   // cos(pi/4)
+    const float2 c1 = make_float2(C1, C1), s1 = make_float2(S1, S1), r2 = make_float2(R2, R2);
+    // position 4 k1 + n2 gets e^{2 pi i n2 k1 / 16}
+    auto eighth = [&](cpk& u) {                   // e^{i pi / 4}
+        const float2 a = sub2(u.r, u.i), b = add2(u.r, u.i);
+        u = {mul2(a, r2), mul2(b, r2)};
+    };
+    auto three_eighths = [&](cpk& u) {            // e^{3 i pi / 4}
+        const float2 a = add2(u.r, u.i), b = sub2(u.r, u.i);
+        u = {mul2(a, neg2(r2)), mul2(b, r2)};
+    };
+    rotate2(v[5], c1, s1);
+    eighth(v[9]);
+    rotate2(v[13], s1, c1);
+    eighth(v[6]);
+    v[10] = {neg2(v[10].i), v[10].r};
+    three_eighths(v[14]);
+    rotate2(v[7], s1, c1);
+    three_eighths(v[11]);
+    rotate2(v[15], neg2(c1), neg2(s1));
+#pragma unroll
+    for (int k1 = 0; k1 < 4; ++k1) dft4_pk(v[4 * k1], v[4 * k1 + 1], v[4 * k1 + 2], v[4 * k1 + 3]);
+}
+
+__device__ __forceinline__ float4 pack4(const cpk& v) { return make_float4(v.r.x, v.r.y, v.i.x, v.i.y); }
+__device__ __forceinline__ cpk unpack4(float4 f) { return {make_float2(f.x, f.y), make_float2(f.z, f.w)}; }
+
+// Hardware barriers: `id` over `count` threads of the CTA (bar.arrive does not
+// wait).  A warp takes part as a whole, so its lanes meet first.
+__device__ __forceinline__ void bar_sync(int id, int count)
+{
+    __syncwarp();
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(int id, int count)
+{
+    __syncwarp();
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
+
+// e^{i pi a / 32} for a compile-time a in [0, 8)
+__device__ __forceinline__ float2 root64(int a)
+{
+    const float C[8] = {1.0f, 0.9951847266721968862448f, 0.9807852804032304491262f, 0.9569403357322088649358f,
+                        0.9238795325112867561282f, 0.8819212643483550297128f, 0.8314696123025452370788f,
+                        0.7730104533627369608109f};
+    const float S[8] = {0.0f, 0.0980171403295606019942f, 0.1950903220161282678483f, 0.2902846772544623676362f,
+                        0.3826834323650897717285f, 0.4713967368259976485564f, 0.5555702330196022247428f,
+                        0.6343932841636454982152f};
+    return make_float2(C[a], S[a]);
+}
+
+// The correlation.  A CTA holds one template's spectra (real route: one row's;
+// pair route: a template's and its partner's) in shared memory, and its two
+// groups of 256 threads take the call's segments in turn, each with a work
+// array of its own: while one group waits at a barrier or for shared memory,
+// the other computes.  A CTA's items (template row, series, segment) are a
+// contiguous share of all of them, so the load is even to one transform
+// whatever the number of rows; a segment's spectrum is read from L2 straight
+// into registers.
+//
+// Spectra are kept as records (see real_spectrum_quads): float4 number
+// (2 r + side) 256 + j (real route) or r 256 + j (pair route) holds, for
+// n = j + 256 r, the bins n and 4096 - n (side 0), 8192 - n and 4096 + n
+// (side 1), as (re, re, im, im).  One record gives Z[n], Z[n + 4096], and their
+// mirrors Z[4096 - n], Z[8192 - n]: the packed inputs n and 4096 - n of the
+// transform.  The second belongs to the thread of 256 - j, which sits 16 lanes
+// away in the same warp: lanes 0-15 of warp w hold j = 16 w + lane, lanes 16-31
+// 256 - j of them (and 128 in the place of 0's, both being their own mirrors).
+//
+// When both groups have formed their last product of a row (barrier EMPTY),
+// the group with the row's last item fetches the next row's spectra during
+// its first two passes and then opens them to the other group (barrier FULL,
+// of two that alternate with the row: the fetching group may reach the next
+// row's before the other has passed this one's).  All waits are hardware
+// barriers between these two groups.
+//
+// What bounds it: the L1/shared-memory pipe, 4.7 K wavefronts a transform (the
+// spectra and norms 1.5 K, the work array 2 K, mirrors 0.3 K), beside 3.8 K
+// cycles of FP32 and 3.2 K of issue; a transform takes 7.3 K cycles.  On 16 s x
+// 4096 templates of 4096 samples (20,480 transforms) it runs 487 us; the form
+// it replaced (one CTA-wide group with the template in registers, unpacked
+// arithmetic, the radix-2 stage last through shared memory, 12.8 K warp
+// instructions more per transform and four CTA-wide barriers) ran 664 us.  The
+// 64 s x 4 series x 65,536 template step went from 163.7 to 121.6 ms.
+template <bool QUAD, bool DENSE>
+__global__ void __launch_bounds__(FT, 1) k_corr_fft(const __grid_constant__ FftParams p, uint32_t total)
+{
+    extern __shared__ __align__(16) float4 csm[];
+    const int g = threadIdx.x / GT, tg = threadIdx.x % GT, warp = tg >> 5, lane = tg & 31;
+    // the transform's input column of this thread, and the lane that holds its mirror
+    const int j = lane < 16 ? 16 * warp + lane : (tg == 16 ? GT / 2 : GT - (16 * warp + lane - 16));
+    const int mate = tg == 0 || tg == 16 ? lane : lane ^ 16;
+    float4* const z = csm + g * ZG;                       // this group's work array
+    float4* const h = csm + 2 * ZG;                       // the template's records [4096]
+    const float2* const twa = reinterpret_cast<const float2*>(h + FH);       // [6][256]
+    const float2* const twb = twa + 6 * GT;               // [15][16]
+    const float4* const twp = reinterpret_cast<const float4*>(twb + 15 * 16);   // [256] pairs
+    float4* const col0 = h + FH + TWC_N / 2 + 9 * g;      // column 0's inputs 2048, 2304 .. 3840, and 0
+    // the warp's reductions over the (row, series) so far, kept out of the registers:
+    // its packed max key (0: none yet; a lag below its value and the tail threshold
+    // changes nothing) and its sum of rho^2
+    struct Acc {
+        unsigned long long best;
+        double ss;
+    };
+    Acc& acc = reinterpret_cast<Acc*>(h + FH + TWC_N / 2 + 2 * 9)[threadIdx.x >> 5];
+    const int BAR_G = 1 + g, BAR_EMPTY = 3, BAR_FULL = 4;          // FULL: two, by the parity of the row
+    constexpr uint32_t BINS = QUAD ? FH : FN;             // complex bins per segment
+    constexpr uint32_t KR = QUAD ? 2 : 1;                 // template rows per item
+
+    const uint32_t n_rows = (p.k_hi - p.k_lo) / KR;
+    // this CTA's items, and its first: segment seg0 of row row0
+    const uint64_t T = (uint64_t)n_rows * total, i0 = T * blockIdx.x / gridDim.x;
+    const uint32_t n_items = (uint32_t)(T * (blockIdx.x + 1) / gridDim.x - i0);
+    if (n_items == 0) return;
+    const uint32_t row0 = (uint32_t)(i0 / total), seg0 = (uint32_t)(i0 % total);
+    const uint32_t row_last = row0 + (uint32_t)(((uint64_t)seg0 + n_items - 1) / total);
+    auto spectra = [&](uint32_t row) {
+        return reinterpret_cast<const float4*>(p.hspec + (size_t)(p.k_lo + row * KR - p.hrow0) * BINS);
+    };
+    {
+        const float4* src = reinterpret_cast<const float4*>(p.tw + TW_N);
+        for (int e = threadIdx.x; e < TWC_N / 2; e += FT) cp_async16(h + FH + e, src + e);
+        src = spectra(row0);
+        for (int e = threadIdx.x; e < FH; e += FT) cp_async16(h + e, src + e);
+        cp_async_commit();
+        if (row0 < row_last) prefetch_l2(reinterpret_cast<const char*>(spectra(row0 + 1)) + 128 * threadIdx.x);
+        cp_async_wait<0>();
+        __syncthreads();
     }
-    if ((threadIdx.x & 31) == 0) {
-        atomicMax(vmax, key);
-        atomicAdd(sumsq, d);
-    }
-}
-
-// The transform of an item in both correlation kernels alternates between the
-// two work arrays, so that no pass waits for the reads of the one before:
-//   product spectrum from x: own bins in registers, mirrors into z   barrier 1
-//   (the next segment's spectrum starts to arrive in x)
-//   pass 1: registers and the mirrors read from z, into z2           barrier 2
-//   pass 2: z2 into z                                                 barrier 3
-//   pass 3: z into z2 (and the next spectrum has arrived)             barrier 4
-//   final radix-2 stage and epilogue read z2.
-// Each array's last reads come before the barrier that precedes its next
-// write: z is read by pass 3 (before barrier 4) and written by the next item's
-// product spectrum; z2 is read by the epilogue and written only after the next
-// item's barrier 1; x is read by the product spectrum and refilled after
-// barrier 1.  Four barriers per item.  The window norms (the per-segment copy,
-// 16-byte aligned rows, carrying 1/F) are read from L2 into registers, half of
-// them while pass 3 runs and half while the first half of the epilogue runs.
-
-// this thread's norms for the lag pairs t = 2 (tid + 512 (I0 + u) + 4096 h),
-// u < 4, of the real route (zero past the segment's nv lags)
-template <int I0>
-__device__ __forceinline__ void load_norm_pairs(const float* __restrict__ nrm, uint32_t nv, float2 (&iv)[8])
-{
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const uint32_t t = 2u * (uint32_t)(threadIdx.x + FT * (I0 + u) + FH * h);
-            iv[2 * u + h] = t < nv ? __ldg(reinterpret_cast<const float2*>(nrm + t)) : make_float2(0.f, 0.f);
-        }
-}
-
-// the same for the lags t = tid + 512 (I0 + u) + 4096 h of the pair route
-template <int I0>
-__device__ __forceinline__ void load_norms(const float* __restrict__ nrm, uint32_t nv, float (&iv)[8])
-{
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const uint32_t t = (uint32_t)(threadIdx.x + FT * (I0 + u) + FH * h);
-            iv[2 * u + h] = t < nv ? __ldg(nrm + t) : 0.f;
-        }
-}
-
-// The correlation of the real route (plain banks).  Each CTA walks its items
-// (template row, series, segment) in order; while the FFT of one segment
-// runs, the spectrum of the next one arrives in shared memory.
-// DENSE: a series of the launch keeps the dense output rho (a compile-time
-// copy, so that the common case carries no per-lag test for it)
-template <bool DENSE>
-__global__ void __launch_bounds__(FT, 1) k_corr_rfft(const __grid_constant__ FftParams p)
-{
-    const Smem m = smem_setup<true>(p.tw);
-    const int tid = threadIdx.x;
-    const float2 base_f = thread_root(4096.0);
-    const float2 base_r = thread_root(8192.0);
-    const uint32_t n_rows = p.k_hi - p.k_lo;
-    uint32_t row = blockIdx.x;
-    if (row >= n_rows || p.n_ser == 0) return;
+    if (g >= (int)n_items) return;                        // a single item: the first group's
+    uint32_t item = g, row = row0, seg = seg0 + g;
     int s = 0;
-    uint32_t j = 0;
-    stage_spectrum<FN>(m, p.ser[0].spec);
-    cp_async_commit();
-    cp_async_wait<0>();
-    __syncthreads();
-
-    float2 hk[FBINS], hp[FBINS], hm = make_float2(0.f, 0.f);
-    uint32_t k = 0;
+    if (seg >= total) {                                   // the second group begins in the next row
+        seg -= total;
+        ++row;
+        bar_arrive(BAR_EMPTY, FT);
+        bar_sync(BAR_FULL + (row & 1), FT);
+    }
+    while (seg >= p.ser[s].nseg) seg -= p.ser[s++].nseg;
+    bool fresh = true;
     float thr = 0.f;
-    // the warp's packed max key over the series so far (0: none yet) and its
-    // value: a lag below both it and the tail threshold changes nothing
-    unsigned long long best = 0ull;
-    float best_v = 0.f;
-    // per-thread sum of rho^2 over a series (a few thousand terms of similar
-    // size: FP32 is ample); the sum over threads is FP64
-    float ss = 0.f;
-    bool new_row = true, new_series = true;
+    // the group's next item, two on
+    auto advance = [&](uint32_t& row, int& s, uint32_t& seg) {
+        seg += 2;
+        while (seg >= p.ser[s].nseg) {
+            seg -= p.ser[s].nseg;
+            if (++s == p.n_ser) {
+                s = 0;
+                ++row;
+            }
+        }
+    };
 
     for (;;) {
         const FftSeries& S = p.ser[s];
-        if (new_row) {
-            k = p.k_lo + row;
-            const float2* H = p.hspec + (size_t)(k - p.hrow0) * FN;
-#pragma unroll
-            for (int i = 0; i < FBINS; ++i) {
-                const int f = tid + FT * i;
-                hk[i] = H[f];
-                hp[i] = H[(FN - f) & (FN - 1)];
-            }
-            if (tid == 0) hm = H[FH];
-        }
-        const uint32_t o = k - p.k_begin;
-        (void)BF_BOUNDS(p.err, o < p.k_end - p.k_begin && k >= p.hrow0 && j < S.nseg);
-        if (new_series) {
+        const uint32_t k = p.k_lo + row * KR;
+        const uint32_t o = (k - p.k_begin) / KR;          // output index
+        (void)BF_BOUNDS(p.err, k + KR - 1 < p.k_end && k >= p.hrow0 && seg < S.nseg);
+        if (fresh) {
             thr = S.sigma_pred ? S.kappa * S.sigma_pred[o] : p.thr;
-            best = 0ull;
-            best_v = 0.f;
-            ss = 0.f;
+            if (lane == 0) acc = Acc{0ull, 0.0};
         }
-        const uint32_t t0 = j * p.V;
+        const uint32_t t0 = seg * p.V;
         const uint32_t nv = min(p.V, S.L - t0);
-        const float* nrm = S.inv + (size_t)j * p.Vp;     // (BF_BOUNDS above: j < nseg)
-        // the item after this one
-        uint32_t np = row, nj = j + 1;
-        int ns = s;
-        if (nj >= S.nseg) {
-            nj = 0;
-            if (++ns >= p.n_ser) {
-                ns = 0;
-                np = row + gridDim.x;
-            }
-        }
-        // Y = X conj(H) over all F bins, and the packed spectrum
-        // Z'[f] = A + i w B, Z'[N - f] = conj(A - i w B), with A = Y[f] +
-        // conj Y[N-f], B = Y[f] - conj Y[N-f], w = e^{i pi f / N}: twice the
-        // transform of c[2n] + i c[2n+1].  The first pass of the FFT reads
-        // Z'[tid + 512 r]: for r < 8 this thread's own, kept in registers; for
-        // r >= 8 those of the mirror thread 512 - tid (thread 0: its own
-        // mirrors and the middle bin), exchanged through shared memory in an
-        // unpadded [8][512] layout of its own: reader j finds Z'[j + 512 r] at
-        // (r - 8) 512 + j, which writer tid fills for its bin r' at
-        // (8 - r') 512 - tid (the middle bin at 0).  A half-warp then writes,
-        // and reads, 16 consecutive values: no bank conflict either way.
-        float vr[16], vi[16];
-#pragma unroll
-        for (int r = 0; r < FBINS; ++r) {
-            const int f = tid + FT * r;
-            if (tid == 0 && r == 0) {
-                // DC and Nyquist (real): Z'[0] = (Y0 + YN) + i (Y0 - YN);
-                // middle bin: Z'[N/2] = 2 conj(Y[N/2]) = 2 conj(X) H
-                const float2 x0 = m.x[0];
-                const float y0 = x0.x * hk[0].x, yn = x0.y * hk[0].y;
-                vr[0] = y0 + yn;
-                vi[0] = y0 - yn;
-                const float2 xm = m.x[FH];
-                m.z[0] = make_float2(2.f * (xm.x * hm.x + xm.y * hm.y), 2.f * (xm.x * hm.y - xm.y * hm.x));
+        const float* nrm = S.inv + (size_t)seg * p.Vp;
+        // Product spectrum and the first radix-2 stage.  Column 0 holds its own
+        // mirrors one place further (256 r goes to 256 (16 - r)), and the record
+        // of n = 0 other bins than the rest: its inputs go through `col0`.
+        cpk v[16];
+        const float4* X = reinterpret_cast<const float4*>(S.spec + (size_t)seg * BINS);
+        if (j == 0) {
+            float zr, zi, mr, mi, er, ei, fr, fi;         // Z[0], Z[4096], Z[2048], Z[6144]
+            if (!QUAD) {
+                // the real bins 0 and 8192 as (re, im) of bin 0, then bins 4096, 6144 and 2048
+                const cpk xk = unpack4(__ldg(X)), xq = unpack4(__ldg(X + GT)), hk = unpack4(h[0]), hq = unpack4(h[GT]);
+                const float y0 = xk.r.x * hk.r.x, yn = xk.i.x * hk.i.x;
+                zr = y0 + yn;
+                zi = y0 - yn;
+                mr = 2.f * (xk.r.y * hk.r.y + xk.i.y * hk.i.y);                  // 2 conj(X) H
+                mi = 2.f * (xk.r.y * hk.i.y - xk.i.y * hk.r.y);
+                const float ykr = xq.r.y * hq.r.y + xq.i.y * hq.i.y, yki = xq.i.y * hq.r.y - xq.r.y * hq.i.y;
+                const float yqr = xq.r.x * hq.r.x + xq.i.x * hq.i.x, yqi = xq.i.x * hq.r.x - xq.r.x * hq.i.x;
+                const float ar = ykr + yqr, ai = yki - yqi, br = ykr - yqr, bi = yki + yqi;
+                constexpr float R2 = 0.707106781186547524f;                     // w = e^{i pi / 4}
+                const float wbr = R2 * (br - bi), wbi = R2 * (br + bi);
+                er = ar - wbi;
+                ei = ai + wbr;
+                fr = ar + wbi;
+                fi = wbr - ai;
             } else {
-                const float2 xk = m.x[f], xq = m.x[FN - f];
-                const float ykr = xk.x * hk[r].x + xk.y * hk[r].y, yki = xk.y * hk[r].x - xk.x * hk[r].y;
-                const float yqr = xq.x * hp[r].x + xq.y * hp[r].y, yqi = xq.y * hp[r].x - xq.x * hp[r].y;
-                const float ar = ykr + yqr, ai = yki - yqi;
-                const float br = ykr - yqr, bi = yki + yqi;
-                const float2 w = cmul(base_r, root32(r));
-                const float wbr = w.x * br - w.y * bi, wbi = w.x * bi + w.y * br;
-                vr[r] = ar - wbi;
-                vi[r] = ai + wbr;
-                m.z[(FBINS - r) * FT - tid] = make_float2(ar + wbi, wbr - ai);
+                // bin 0 holds the real bins 0 and 4096; the other lane bin 2048
+                const cpk x = unpack4(__ldg(X)), ha = unpack4(h[0]), hb = unpack4(h[FH / 2]);
+                zr = x.r.x * ha.r.x;
+                zi = x.r.x * hb.r.x;
+                mr = x.i.x * ha.i.x;
+                mi = x.i.x * hb.i.x;
+                const float yar = x.r.y * ha.r.y + x.i.y * ha.i.y, yai = x.i.y * ha.r.y - x.r.y * ha.i.y;
+                const float ybr = x.r.y * hb.r.y + x.i.y * hb.i.y, ybi = x.i.y * hb.r.y - x.r.y * hb.i.y;
+                er = yar - ybi;
+                ei = yai + ybr;
+                fr = yar + ybi;
+                fi = ybr - yai;
+            }
+            col0[8] = make_float4(zr + mr, zr - mr, zi + mi, zi - mi);          // the input 0
+            col0[0] = make_float4(er + fr, fi - ei, ei + fi, er - fr);          // the input 2048, twiddle i
+        }
+        const float4 roots = twp[j];
+        const float2 base_w = make_float2(roots.x, roots.y), base_t = make_float2(roots.z, roots.w);
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            const float2 w = r ? cmul(base_w, root64(r)) : base_w;          // e^{i pi n / 8192}
+            const float2 t = r ? cmul(base_t, root32(r)) : base_t;          // e^{2 pi i n / 8192}
+            float2 pr, pi, qr, qi;          // (Z[n], Z[4096 - n]) and (Z[8192 - n], Z[4096 + n])
+            if (!QUAD) {
+                const cpk xk = unpack4(__ldg(X + 2 * r * GT + j)), xq = unpack4(__ldg(X + (2 * r + 1) * GT + j));
+                const cpk hk = unpack4(h[2 * r * GT + j]), hq = unpack4(h[(2 * r + 1) * GT + j]);
+                const float2 wr = make_float2(w.x, w.y), wi = make_float2(w.y, w.x);     // lanes n, 4096 - n
+                const float2 ykr = fma2(xk.r, hk.r, mul2(xk.i, hk.i)), yki = fma2(xk.i, hk.r, neg2(mul2(xk.r, hk.i)));
+                const float2 yqr = fma2(xq.r, hq.r, mul2(xq.i, hq.i)), yqi = fma2(xq.i, hq.r, neg2(mul2(xq.r, hq.i)));
+                // A = Y[k] + conj Y[N-k], B = Y[k] - conj Y[N-k], Z[k] = A + i w B, Z[N-k] = conj(A - i w B)
+                const float2 ar = add2(ykr, yqr), ai = sub2(yki, yqi), br = sub2(ykr, yqr), bi = add2(yki, yqi);
+                const float2 wbr = fma2(wr, br, neg2(mul2(wi, bi))), wbi = fma2(wr, bi, mul2(wi, br));
+                pr = sub2(ar, wbi);
+                pi = add2(ai, wbr);
+                qr = add2(ar, wbi);
+                qi = sub2(wbr, ai);
+            } else {
+                const cpk x = unpack4(__ldg(X + r * GT + j));
+                const cpk ha = unpack4(h[r * GT + j]), hb = unpack4(h[FH / 2 + r * GT + j]);
+                const float2 yar = fma2(x.r, ha.r, mul2(x.i, ha.i)), yai = fma2(x.i, ha.r, neg2(mul2(x.r, ha.i)));
+                const float2 ybr = fma2(x.r, hb.r, mul2(x.i, hb.i)), ybi = fma2(x.i, hb.r, neg2(mul2(x.r, hb.i)));
+                // Z = Ya + i Yb, Z[N - k] = conj(Ya) + i conj(Yb)
+                pr = sub2(yar, ybi);
+                pi = add2(yai, ybr);
+                qr = add2(yar, ybi);
+                qi = sub2(ybr, yai);
+            }
+            // input n: from Z[n] and Z[n + 4096], twiddle t; input 4096 - n: from
+            // Z[4096 - n] and Z[8192 - n], twiddle -conj(t)
+            const float dr = pr.x - qr.y, di = pi.x - qi.y, er = pr.y - qr.x, ei = pi.y - qi.x;
+            v[r] = {make_float2(pr.x + qr.y, dr * t.x - di * t.y), make_float2(pi.x + qi.y, dr * t.y + di * t.x)};
+            const float4 f = make_float4(pr.y + qr.x, -er * t.x - ei * t.y, pi.y + qi.x, er * t.y - ei * t.x);
+            if (r > 0 && j == 0) col0[8 - r] = f;
+            v[15 - r] = {make_float2(__shfl_sync(0xffffffffu, f.x, mate), __shfl_sync(0xffffffffu, f.y, mate)),
+                         make_float2(__shfl_sync(0xffffffffu, f.z, mate), __shfl_sync(0xffffffffu, f.w, mate))};
+        }
+        if (j == 0) {
+            v[0] = unpack4(col0[8]);
+#pragma unroll
+            for (int r = 0; r < 8; ++r) v[8 + r] = unpack4(col0[r]);
+        }
+        // this group's last product of the row: the spectra may be replaced
+        const bool more = item + 2 < n_items;
+        bool loading = false, departed = false;
+        if (row < row_last) {
+            uint32_t nrow = row, nseg = seg;
+            int ns = s;
+            advance(nrow, ns, nseg);
+            if (more && nrow == row) {
+                // not the last
+            } else if ((((row - row0 + 1) * total - seg0 - 1) & 1) == (uint32_t)g) {       // the row's last item is this group's
+                bar_sync(BAR_EMPTY, FT);
+                const float4* src = spectra(row + 1);
+#pragma unroll
+                for (int e = 0; e < FH / GT; ++e) cp_async16(h + e * GT + tg, src + e * GT + tg);
+                cp_async_commit();
+                if (row + 2 <= row_last) {                // the row after into L2 (64 KiB)
+                    const char* nx = reinterpret_cast<const char*>(spectra(row + 2));
+                    prefetch_l2(nx + 256 * tg);
+                    prefetch_l2(nx + 256 * tg + 128);
+                }
+                loading = true;
+            } else {
+                bar_arrive(BAR_EMPTY, FT);
+                departed = true;
             }
         }
-        __syncthreads();                            // 1
-        if (np < n_rows) stage_spectrum<FN>(m, p.ser[ns].spec + (size_t)nj * FN);
-        cp_async_commit();
-        if (np != row && np < n_rows)               // the next row's template spectrum into L2 (64 KiB)
-            prefetch_l2(p.hspec + (size_t)(p.k_lo + np - p.hrow0) * FN + 16 * tid);
+        // pass 1: out k0 = q at position 4 k1 + k2 of dft16, q = k1 + 4 k2; twiddle e^{2 pi i q j / 4096}
+        dft16_pk(v);
+        {
+            float2 w[4], u[4];
 #pragma unroll
-        for (int r = FBINS; r < 16; ++r) {
-            const float2 v = m.z[(r - FBINS) * FT + tid];
-            vr[r] = v.x;
-            vi[r] = v.y;
-        }
-        pass16_from<1, 1>(m, m.z2, vr, vi);               // 2
-        pass16<1, 16, -1, false>(m, m.z2, m.z);           // 3
-        float2 iv0[8], iv1[8];
-        load_norm_pairs<0>(nrm, nv, iv0);
-        pass16<1, 256, 0, false>(m, m.z, m.z2);           // 4, and the next segment's spectrum
-        load_norm_pairs<4>(nrm, nv, iv1);
-        float pa = 0.f;
-        // lag pairs t = 2 (tid + 512 i + 4096 h) for i = i0 + u, with norms iv
-        auto lags = [&](const int i0, const float2 (&iv)[8]) {
+            for (int e = 1; e < 4; ++e) {
+                w[e] = twa[(e - 1) * GT + j];             // q = 1, 2, 3
+                u[e] = twa[(e + 2) * GT + j];             // q = 4, 8, 12
+            }
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int i = i0 + u;
-                float2 w = final_tw<1>(base_f, u);     // e^{i pi (tid + 512 u) / 4096} ...
-                if (i0) w = make_float2(-w.y, w.x);    // ... times e^{i pi / 2} for i = 4 + u
-                float2 z[2];
-                fft_final(m.z2, i, w, z[0], z[1]);
-                // z = c[2n] + i c[2n + 1]: the lag pairs t = 2 (tid + 512 i + 4096 h);
-                // norms carry 1/F (k_fft_flags), and the norm of t + 1 is 0 when t
-                // is the segment's last lag, so rb is 0 there
-                float ra[2], rb[2], g = 0.f;
+            for (int k2 = 0; k2 < 4; ++k2)
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const uint32_t t = 2u * (uint32_t)(tid + FT * i + FH * h);
-                    ra[h] = rb[h] = 0.f;
-                    if (t < nv) {
-                        ra[h] = z[h].x * iv[2 * u + h].x;
-                        rb[h] = z[h].y * iv[2 * u + h].y;
-                        if (DENSE && S.rho) {
-                            const uint32_t tau = t0 + t;
-                            const bool two = t + 1 < nv;
-                            if (BF_BOUNDS(p.err, tau + (two ? 1u : 0u) < S.L)) {
-                                S.rho[(size_t)o * S.L + tau] = ra[h];
-                                if (two) S.rho[(size_t)o * S.L + tau + 1] = rb[h];
-                            }
-                        }
-                    }
-                    pa = fmaf(ra[h], ra[h], pa);
-                    pa = fmaf(rb[h], rb[h], pa);
-                    g = fmaxf(g, fmaxf(fabsf(ra[h]), fabsf(rb[h])));
+                for (int k1 = 0; k1 < 4; ++k1) {
+                    if (k1 + k2 == 0) continue;
+                    const float2 f = k1 == 0 ? u[k2] : k2 == 0 ? w[k1] : cmul(u[k2], w[k1]);
+                    rotate2(v[4 * k1 + k2], make_float2(f.x, f.x), make_float2(f.y, f.y));
                 }
-                // only lags reaching the warp's running max (ties included: an
-                // earlier lag wins them) or the tail threshold need their keys
-                if (warp_max_abs(g) >= fminf(thr, best_v)) {
-                    unsigned long long lk = 0ull;
+            bar_sync(BAR_G, GT);                          // 1: every warp is done with the work array
+            float4* const zz = z + (j >> 4) * ZROW + (j & 15);
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const uint32_t t = 2u * (uint32_t)(tid + FT * i + FH * h);
-                        if (t < nv) {
-                            const uint32_t tau = t0 + t;
-                            const float aa = fabsf(ra[h]), ab = fabsf(rb[h]);
-                            // the pair's larger |rho|, the earlier lag on ties
-                            const bool second = ab > aa;
-                            track_max(second ? ab : aa, second ? tau + 1 : tau, lk);
-                            if (fmaxf(aa, ab) >= thr) {
-                                if (aa >= thr) push_tail(p, S.series_id, k, tau, ra[h]);
-                                if (t + 1 < nv && ab >= thr) push_tail(p, S.series_id, k, tau + 1, rb[h]);
-                            }
-                        }
-                    }
-                    lk = warp_max_key(lk);
-                    best = lk > best ? lk : best;
-                    best_v = __uint_as_float((uint32_t)(best >> 32));
+            for (int c = 0; c < 16; ++c) zz[((c >> 2) + 4 * (c & 3)) * ZBLK] = pack4(v[c]);
+        }
+        bar_sync(BAR_G, GT);                              // 2: pass 1 is written
+        {
+            // pass 2: thread (k0, n0) = (tg / 16, tg % 16); twiddle e^{2 pi i q n0 / 256}
+            float4* const zz = z + (tg >> 4) * ZBLK + (tg & 15);
+#pragma unroll
+            for (int r = 0; r < 16; ++r) v[r] = unpack4(zz[ZROW * r]);
+            dft16_pk(v);
+#pragma unroll
+            for (int c = 0; c < 16; ++c) {
+                const int q = (c >> 2) + 4 * (c & 3);
+                if (q) {
+                    const float2 f = twb[(q - 1) * 16 + (tg & 15)];
+                    rotate2(v[c], make_float2(f.x, f.x), make_float2(f.y, f.y));
+                }
+                zz[ZROW * q] = pack4(v[c]);
+            }
+        }
+        if (loading) {
+            cp_async_wait<0>();                           // this thread's part of the next row's spectra
+            bar_arrive(BAR_FULL + ((row + 1) & 1), FT);
+        }
+        __syncwarp();
+        // pass 3: thread (k0, k1) = (tg / 16, tg % 16); output k = k0 + 16 k1 + 256 q
+        {
+            const float4* const zz = z + (tg >> 4) * ZBLK + (tg & 15) * ZROW;
+#pragma unroll
+            for (int r = 0; r < 16; ++r) v[r] = unpack4(zz[r]);
+        }
+        // norms of the lags of this thread's output q: lags 4 k .. 4 k + 3 in the order
+        // 0, 2, 1, 3 (real route), lags 2 k, 2 k + 1 (pair route), stored by (q, tg);
+        // zero past the segment's end
+        auto norms = [&](int q) -> float4 {
+            if ((QUAD ? 2u : 4u) * GT * q >= nv) return make_float4(0.f, 0.f, 0.f, 0.f);
+            if (!QUAD) return __ldg(reinterpret_cast<const float4*>(nrm) + GT * q + tg);
+            const float2 f = __ldg(reinterpret_cast<const float2*>(nrm) + GT * q + tg);
+            return make_float4(f.x, f.y, 0.f, 0.f);
+        };
+        constexpr int AHEAD = 6;
+        float4 iv[AHEAD];
+#pragma unroll
+        for (int q = 0; q < AHEAD; ++q) iv[q] = norms(q);
+        dft16_pk(v);
+        // rho in place, the sum of its squares and this thread's largest |rho|
+        float2 pa = make_float2(0.f, 0.f);
+        float m = 0.f;
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+            // past the segment's lags (at M = 4096 half of the pair route's outputs;
+            // the real route's, a fifth at most, cost less than the branches would)
+            if (QUAD && q >= 4 && 2u * GT * q >= nv) continue;
+            cpk& c = v[4 * (q & 3) + (q >> 2)];
+            const float4 n = iv[q % AHEAD];
+            if (q + AHEAD < 16) iv[q % AHEAD] = norms(q + AHEAD);
+            if (!QUAD) {
+                c.r = mul2(c.r, make_float2(n.x, n.y));           // lags t, t + 2
+                c.i = mul2(c.i, make_float2(n.z, n.w));           // lags t + 1, t + 3
+                pa = fma2(c.r, c.r, pa);
+                pa = fma2(c.i, c.i, pa);
+                m = fmaxf(m, fmaxf(fabsf(c.r.x), fabsf(c.r.y)));
+                m = fmaxf(m, fmaxf(fabsf(c.i.x), fabsf(c.i.y)));
+            } else {
+                const float2 e = fma2(c.r, c.r, mul2(c.i, c.i));
+                c.r = mul2(make_float2(sqrtf(e.x), sqrtf(e.y)), make_float2(n.x, n.y));
+                pa = fma2(c.r, c.r, pa);
+                m = fmaxf(m, fmaxf(c.r.x, c.r.y));
+            }
+        }
+        // f(lag in the segment, rho) over this thread's lags in increasing order
+        auto each = [&](auto f) {
+#pragma unroll
+            for (int q = 0; q < 16; ++q) {
+                const cpk& c = v[4 * (q & 3) + (q >> 2)];
+                const uint32_t t = (QUAD ? 2u : 4u) * (uint32_t)((tg >> 4) + 16 * (tg & 15) + GT * q);
+                f(t, c.r.x);
+                f(t + 1, QUAD ? c.r.y : c.i.x);
+                if (!QUAD) {
+                    f(t + 2, c.r.y);
+                    f(t + 3, c.i.y);
                 }
             }
         };
-        lags(0, iv0);
-        lags(4, iv1);
-        ss += pa;
-        if (nj == 0)                                // last segment of this series: publish
-            publish(best, (double)ss, S.vmax + o, S.sumsq + o);
-        if (np >= n_rows) break;
-        new_row = np != row;
-        new_series = nj == 0;
-        row = np;
-        s = ns;
-        j = nj;
-    }
-}
-
-// The correlation of the pair route (quadrature banks): a template and its
-// quadrature partner in one complex transform, |rho| = |c_cos + i c_sin| /
-// |window|.  Each CTA walks its items (pair, series, segment) in order, with
-// the next segment's spectrum staged and the norms read as above.  DENSE as
-// in k_corr_rfft.
-template <bool DENSE>
-__global__ void __launch_bounds__(FT, 1) k_corr_fft_quad(const __grid_constant__ FftParams p)
-{
-    const Smem m = smem_setup<true>(p.tw);
-    const int tid = threadIdx.x;
-
-    const float2 base_f = thread_root(4096.0);
-    const uint32_t n_pairs = (p.k_hi - p.k_lo + 1) / 2;
-    uint32_t pair = blockIdx.x;
-    if (pair >= n_pairs || p.n_ser == 0) return;
-    int s = 0;
-    uint32_t j = 0;
-    stage_spectrum<FH>(m, p.ser[0].spec);
-    cp_async_commit();
-    cp_async_wait<0>();
-    __syncthreads();
-
-    float2 ha[FBINS], hb[FBINS];
-    uint32_t ka = 0;
-    float thr = 0.f;
-    unsigned long long best = 0ull;             // the warp's packed max key, as above
-    float best_v = 0.f;
-    float ss = 0.f;
-    bool new_pair = true, new_series = true;
-
-    for (;;) {
-        const FftSeries& S = p.ser[s];
-        if (new_pair) {
-            ka = p.k_lo + 2 * pair;
-#pragma unroll
-            for (int i = 0; i < FBINS; ++i) {
-                const int f = tid + FT * i;
-                ha[i] = p.hspec[(size_t)(ka - p.hrow0) * FH + f];
-                hb[i] = p.hspec[(size_t)(ka + 1 - p.hrow0) * FH + f];
+        if (DENSE && S.rho)
+            each([&](uint32_t t, float r) {
+                if (t < nv && BF_BOUNDS(p.err, t0 + t < S.L)) S.rho[(size_t)o * S.L + t0 + t] = r;
+            });
+        // only a warp whose largest |rho| reaches its running max (ties
+        // included: an earlier lag wins them) or the tail threshold looks at
+        // single lags
+        m = warp_max_abs(m);
+        __syncwarp();
+        const float best_v = __uint_as_float((uint32_t)(acc.best >> 32));
+        if (m >= fminf(thr, best_v)) {
+            if (m >= best_v) {
+                // the earliest lag that has it (a padded lag has rho = 0 and a
+                // later lag than the segment's: it cannot win)
+                uint32_t first = 0xffffffffu;
+                each([&](uint32_t t, float r) {
+                    if (fabsf(r) == m) first = min(first, t);
+                });
+                first = __reduce_min_sync(0xffffffffu, first);
+                const unsigned long long key = pack_max(m, t0 + first);
+                if (lane == 0 && key > acc.best) acc.best = key;
             }
+            if (m >= thr)
+                each([&](uint32_t t, float r) {
+                    if (t < nv && fabsf(r) >= thr) push_tail(p, S.series_id, QUAD ? k >> 1 : k, t0 + t, r);
+                });
         }
-        const uint32_t la = (ka - p.k_begin) >> 1;           // output index of the pair
-        (void)BF_BOUNDS(p.err, ka + 1 < p.k_end && ka >= p.hrow0 && j < S.nseg);
-        if (new_series) {
-            thr = S.sigma_pred ? S.kappa * S.sigma_pred[la] : p.thr;
-            best = 0ull;
-            best_v = 0.f;
-            ss = 0.f;
-        }
-        const uint32_t t0 = j * p.V;
-        const uint32_t nv = min(p.V, S.L - t0);
-        const float* nrm = S.inv + (size_t)j * p.Vp;
-        uint32_t np = pair, nj = j + 1;
+        float sum = pa.x + pa.y;                          // 64 terms of a thread, then 32 threads
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+        if (lane == 0) acc.ss += (double)sum;
+        uint32_t nrow = row;
         int ns = s;
-        if (nj >= S.nseg) {
-            nj = 0;
-            if (++ns >= p.n_ser) {
-                ns = 0;
-                np = pair + gridDim.x;
-            }
+        asm volatile("" : "+r"(seg));                     // recomputed here, not kept in registers
+        advance(nrow, ns, seg);
+        fresh = !more || ns != s || nrow != row;
+        if (fresh && lane == 0) {
+            atomicMax(S.vmax + o, acc.best);
+            atomicAdd(S.sumsq + o, acc.ss);
         }
-        // Z = X conj(H_a) + i X conj(H_b); Z[F - f] = conj(Ya) + i conj(Yb),
-        // exchanged with the mirror thread as in k_corr_rfft
-        float vr[16], vi[16];
-#pragma unroll
-        for (int i = 0; i < FBINS; ++i) {
-            const float2 x = m.x[tid + FT * i];
-            if (tid == 0 && i == 0) {
-                // DC (x.x) and Nyquist (x.y): real products
-                vr[0] = x.x * ha[0].x;
-                vi[0] = x.x * hb[0].x;
-                m.z[0] = make_float2(x.y * ha[0].y, x.y * hb[0].y);
-            } else {
-                const float yar = x.x * ha[i].x + x.y * ha[i].y;
-                const float yai = x.y * ha[i].x - x.x * ha[i].y;
-                const float ybr = x.x * hb[i].x + x.y * hb[i].y;
-                const float ybi = x.y * hb[i].x - x.x * hb[i].y;
-                vr[i] = yar - ybi;
-                vi[i] = yai + ybr;
-                m.z[(FBINS - i) * FT - tid] = make_float2(yar + ybi, ybr - yai);
-            }
+        if (!more) break;
+        // the spectra of the next item's row: fetched by this group (all its
+        // threads' parts) or by the other
+        if (loading) {
+            bar_sync(BAR_G, GT);
+            ++row;
         }
-        __syncthreads();                            // 1
-        if (np < n_pairs) stage_spectrum<FH>(m, p.ser[ns].spec + (size_t)nj * FH);
-        cp_async_commit();
-        if (np != pair && np < n_pairs)             // the next pair's two spectra into L2 (64 KiB)
-            prefetch_l2(p.hspec + (size_t)(p.k_lo + 2 * np - p.hrow0) * FH + 16 * tid);
-#pragma unroll
-        for (int r = FBINS; r < 16; ++r) {
-            const float2 v = m.z[(r - FBINS) * FT + tid];
-            vr[r] = v.x;
-            vi[r] = v.y;
+        while (row < nrow) {
+            if (!departed) bar_arrive(BAR_EMPTY, FT);
+            ++row;
+            bar_sync(BAR_FULL + (row & 1), FT);
+            departed = false;
         }
-        pass16_from<1, 1>(m, m.z2, vr, vi);               // 2
-        pass16<1, 16, -1, false>(m, m.z2, m.z);           // 3
-        float iv0[8], iv1[8];
-        load_norms<0>(nrm, nv, iv0);
-        pass16<1, 256, 0, false>(m, m.z, m.z2);           // 4, and the next segment's spectrum
-        load_norms<4>(nrm, nv, iv1);
-        float pa = 0.f;
-        auto lags = [&](const int i0, const float (&iv)[8]) {
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int i = i0 + u;
-                float2 w = final_tw<1>(base_f, u);
-                if (i0) w = make_float2(-w.y, w.x);
-                float2 z[2];
-                fft_final(m.z2, i, w, z[0], z[1]);
-                float r[2];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const uint32_t t = (uint32_t)(tid + FT * i + FH * h);
-                    r[h] = 0.f;
-                    if (t < nv) {
-                        const uint32_t tau = t0 + t;
-                        r[h] = sqrtf(z[h].x * z[h].x + z[h].y * z[h].y) * iv[2 * u + h];   // norms carry 1/F
-                        pa = fmaf(r[h], r[h], pa);
-                        if (DENSE && S.rho && BF_BOUNDS(p.err, tau < S.L)) S.rho[(size_t)la * S.L + tau] = r[h];
-                    }
-                }
-                if (warp_max_abs(fmaxf(r[0], r[1])) >= fminf(thr, best_v)) {
-                    unsigned long long lk = 0ull;
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const uint32_t t = (uint32_t)(tid + FT * i + FH * h);
-                        if (t < nv) {
-                            track_max(r[h], t0 + t, lk);
-                            if (r[h] >= thr) push_tail(p, S.series_id, ka >> 1, t0 + t, r[h]);
-                        }
-                    }
-                    lk = warp_max_key(lk);
-                    best = lk > best ? lk : best;
-                    best_v = __uint_as_float((uint32_t)(best >> 32));
-                }
-            }
-        };
-        lags(0, iv0);
-        lags(4, iv1);
-        ss += pa;
-        if (nj == 0)
-            publish(best, (double)ss, S.vmax + la, S.sumsq + la);
-        if (np >= n_pairs) break;
-        new_pair = np != pair;
-        new_series = nj == 0;
-        pair = np;
+        item += 2;
         s = ns;
-        j = nj;
     }
 }
 
@@ -1090,9 +1218,12 @@ __global__ void __launch_bounds__(FT, 1) k_corr_fft_quad(const __grid_constant__
 // energies come from the FP64 prefix of x^2.  One grid row per series.
 // Every norm is also written, times the inverse transform's scale (a power of
 // two, so exactly), to the per-segment copy the correlation kernel reads:
-// segment j's lags at inv_seg[j Vp ..), Vp = V rounded up to a multiple of 4,
+// segment j's lags at inv_seg[j Vp ..), Vp = V rounded up as said below,
 // so every segment starts 16-byte aligned; past a segment's last lag its row
-// holds zeros, so that the real route reads whole pairs (t, t + 1) of norms.
+// holds zeros.  Inside a row the norms stand as the threads of the correlation
+// kernel's last pass read them: outputs k = k0 + 16 k1 + 256 q in the order (q, k0,
+// k1), each with its lags 4 k, 4 k + 2, 4 k + 1, 4 k + 3 (real route) or 2 k, 2 k + 1
+// (pair route); Vp is V rounded up to whole q.
 __global__ void __launch_bounds__(256) k_fft_flags(const __grid_constant__ FftSeriesBatch b)
 {
     const int i = blockIdx.y;
@@ -1101,6 +1232,12 @@ __global__ void __launch_bounds__(256) k_fft_flags(const __grid_constant__ FftSe
     const double* S = b.S[i];
     float* inv = b.inv[i];
     const uint32_t lane = threadIdx.x & 31;
+    // the place of lag u of a segment in its row
+    auto place = [&](uint64_t u) -> uint64_t {
+        const uint64_t k = b.quad ? u >> 1 : u >> 2;
+        const uint64_t at = (k & ~255ull) | ((k & 15) << 4) | ((k >> 4) & 15);
+        return b.quad ? 2 * at + (u & 1) : 4 * at + ((u & 1) << 1 | ((u >> 1) & 1));
+    };
     {
         // the zeros: Vp - V per full segment, Vp - (its lags) in the last one
         const uint64_t nseg = (L + b.V - 1) / b.V;
@@ -1109,8 +1246,8 @@ __global__ void __launch_bounds__(256) k_fft_flags(const __grid_constant__ FftSe
         const uint64_t n_pad = n_full + (b.Vp - last);
         for (uint64_t q = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; q < n_pad;
              q += (uint64_t)gridDim.x * blockDim.x) {
-            const uint64_t pos = q < n_full ? (q / padv) * b.Vp + b.V + q % padv
-                                            : (nseg - 1) * b.Vp + last + (q - n_full);
+            const uint64_t pos = q < n_full ? (q / padv) * b.Vp + place(b.V + q % padv)
+                                            : (nseg - 1) * b.Vp + place(last + (q - n_full));
             if (BF_BOUNDS(b.err, pos < nseg * b.Vp)) b.inv_seg[i][pos] = 0.f;
         }
     }
@@ -1129,7 +1266,7 @@ __global__ void __launch_bounds__(256) k_fft_flags(const __grid_constant__ FftSe
                 const double E = S[e] - S[a];
                 flag = E * (double)iv * (double)iv > FFT_FIX_RATIO2;
             }
-            b.inv_seg[i][j * b.Vp + (t - a)] = flag ? 0.f : iv * b.scale;
+            b.inv_seg[i][j * b.Vp + place(t - a)] = flag ? 0.f : iv * b.scale;
         }
         const uint32_t mask = __ballot_sync(0xffffffffu, flag);
         if (mask == 0u) continue;
@@ -1275,19 +1412,19 @@ cudaError_t fft_attributes()
 {
     static bool done = false;
     if (done) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(k_corr_rfft<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RCORR_SMEM);
+    cudaError_t e = cudaFuncSetAttribute(k_corr_fft<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CORR_SMEM);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_corr_rfft<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RCORR_SMEM);
+        e = cudaFuncSetAttribute(k_corr_fft<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CORR_SMEM);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_corr_fft_quad<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CORR_SMEM);
+        e = cudaFuncSetAttribute(k_corr_fft<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CORR_SMEM);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_corr_fft_quad<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CORR_SMEM);
+        e = cudaFuncSetAttribute(k_corr_fft<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CORR_SMEM);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_fft_series<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FFT_SMEM);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_fft_series<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FFT_SMEM);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_fft_bank_real, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CORR_SMEM);
+        e = cudaFuncSetAttribute(k_fft_bank_real, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BANK_SMEM);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_fft_bank_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FFT_SMEM);
     if (e == cudaSuccess)
@@ -1309,7 +1446,7 @@ cudaError_t fft_tables(bf_ctx* ctx, cudaStream_t st, const float2** out)
 {
     if (!ctx->fft_tw) {
         float2* t = nullptr;
-        cudaError_t e = cudaMalloc(&t, TW_N * sizeof(float2));
+        cudaError_t e = cudaMalloc(&t, (TW_N + TWC_N) * sizeof(float2));
         if (e != cudaSuccess) return e;
         count_launches(1);
         k_fft_tables<<<(TW_N + 255) / 256, 256, 0, st>>>(t);
@@ -1350,7 +1487,7 @@ static cudaError_t template_spectra(const bf_bank* bank, size_t row0, size_t nro
         const unsigned grid = std::min<uint32_t>(items, (uint32_t)n_sm);
         count_launches(1);
         if (bank->quad) k_fft_bank_pair<<<grid, FT, FFT_SMEM, st>>>(scratch, (uint32_t)kc, items, tw, out + k * bins);
-        else k_fft_bank_real<<<grid, FT, CORR_SMEM, st>>>(scratch, (uint32_t)kc, bank->M, tw, out + k * bins);
+        else k_fft_bank_real<<<grid, FT, BANK_SMEM, st>>>(scratch, (uint32_t)kc, bank->M, tw, out + k * bins);
         e = cudaGetLastError();
     }
     return e;
@@ -1399,7 +1536,11 @@ bf_status bank_fft_spectra(bf_ctx* ctx, bf_bank* bank, cudaStream_t st)
 }
 
 uint32_t fft_lags_per_seg(uint32_t M, bool quad) { return fft_seg_len(quad) - M + 1; }
-uint32_t fft_norm_stride(uint32_t M, bool quad) { return (fft_lags_per_seg(M, quad) + 3) & ~3u; }
+uint32_t fft_norm_stride(uint32_t M, bool quad)
+{
+    const uint32_t q = (quad ? 2 : 4) * GT;          // lags of one output of every thread
+    return (fft_lags_per_seg(M, quad) + q - 1) / q * q;
+}
 // 1/F for the real route: the inverse transform is unnormalised and the
 // even/odd split forms twice the packed spectrum; 1/N for the pair route
 float fft_inverse_scale(bool quad) { return 1.f / (float)fft_seg_len(quad); }
@@ -1466,18 +1607,26 @@ cudaError_t launch_fft_series(const FftSeriesBatch& b, uint32_t total_segments, 
 
 cudaError_t launch_corr_fft(const FftParams& p, int n_sm, cudaStream_t st)
 {
-    const uint32_t items = p.quad ? (p.k_hi - p.k_lo + 1) / 2 : p.k_hi - p.k_lo;
-    if (items == 0 || p.n_ser == 0) return cudaSuccess;
-    const unsigned grid = std::min<unsigned>(items, (unsigned)n_sm);
-    count_launches(1);
+    const uint32_t rows = p.quad ? (p.k_hi - p.k_lo) / 2 : p.k_hi - p.k_lo;
+    if (rows == 0 || p.n_ser == 0) return cudaSuccess;
+    uint64_t total = 0;                       // segments of a row
     bool dense = false;
-    for (int i = 0; i < p.n_ser; ++i) dense = dense || p.ser[i].rho != nullptr;
+    for (int i = 0; i < p.n_ser; ++i) {
+        total += p.ser[i].nseg;
+        dense = dense || p.ser[i].rho != nullptr;
+    }
+    if (total == 0 || total > 0x7FFFFFFFull) return cudaErrorInvalidValue;
+    // contiguous shares of the rows x total transforms: a CTA needs one at least,
+    // and counts its own in 32 bits
+    const uint64_t T = rows * total;
+    const unsigned grid = (unsigned)std::min<uint64_t>(T, std::max<uint64_t>((uint64_t)n_sm, T >> 30));
+    count_launches(1);
     if (p.quad) {
-        if (dense) k_corr_fft_quad<true><<<grid, FT, CORR_SMEM, st>>>(p);
-        else k_corr_fft_quad<false><<<grid, FT, CORR_SMEM, st>>>(p);
+        if (dense) k_corr_fft<true, true><<<grid, FT, CORR_SMEM, st>>>(p, (uint32_t)total);
+        else k_corr_fft<true, false><<<grid, FT, CORR_SMEM, st>>>(p, (uint32_t)total);
     } else {
-        if (dense) k_corr_rfft<true><<<grid, FT, RCORR_SMEM, st>>>(p);
-        else k_corr_rfft<false><<<grid, FT, RCORR_SMEM, st>>>(p);
+        if (dense) k_corr_fft<false, true><<<grid, FT, CORR_SMEM, st>>>(p, (uint32_t)total);
+        else k_corr_fft<false, false><<<grid, FT, CORR_SMEM, st>>>(p, (uint32_t)total);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || !p.chirps) return e;
