@@ -642,12 +642,17 @@ size_t result_bytes(const bf_bank* bank, const bf_opts& o, size_t N, double fs, 
 cudaError_t clear_result(bf_result* r, cudaStream_t st)
 {
     const size_t S = r->n_series, K = r->K;
-    cudaError_t e = cudaMemsetAsync(r->packed, 0, S * K * 8, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(r->sumsq, 0, S * K * 8, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(r->cand_count, 0, 2 * sizeof(unsigned int), st);
-    if (e == cudaSuccess && r->hist) e = cudaMemsetAsync(r->hist, 0, S * r->nbins * 4, st);
-    if (e == cudaSuccess && r->map) e = cudaMemsetAsync(r->map, 0, r->map_total * 4, st);
-    return e;
+    ClearParams p{};
+    auto add = [&p](void* a, size_t bytes) {
+        p.ptr[p.n] = static_cast<uint32_t*>(a);
+        p.words[p.n++] = bytes / 4;
+    };
+    add(r->packed, S * K * 8);
+    add(r->sumsq, S * K * 8);
+    add(r->cand_count, 2 * sizeof(unsigned int));
+    if (r->hist) add(r->hist, S * r->nbins * 4);
+    if (r->map) add(r->map, r->map_total * 4);
+    return launch_clear(p, st);
 }
 
 // Finalize kernels for a result whose correlation launches are enqueued.

@@ -274,7 +274,7 @@ struct PrepBatch {
     uint64_t N[MAX_PREP];
     uint64_t xcap[MAX_PREP];
     uint64_t nb[MAX_PREP];          // FP64 scan blocks of the series
-    double* bsum[MAX_PREP];         // their sums: 2 nb doubles (energies, counts)
+    double* bsum[MAX_PREP];         // their sums: nb doubles (energies), then nb counts (32-bit)
     double* S[MAX_PREP];            // prefix of x^2 [N + 1], then the uint32 counts [N + 1]
     float* inv[MAX_PREP];           // [N - M + 1]
     unsigned int* status[MAX_PREP];
@@ -313,6 +313,14 @@ struct FinalizeSeries {
     uint32_t L;
     uint32_t nt;
 };
+// arrays of 32-bit words, 16-byte aligned, zeroed by one launch
+struct ClearParams {
+    int n;
+    uint32_t* ptr[5];
+    uint64_t words[5];
+};
+cudaError_t launch_clear(const ClearParams& p, cudaStream_t s);
+
 constexpr int MAX_FIN = 128;        // series per finalize / paint launch
 struct FinalizeParams {
     uint32_t s0, n;                 // series [s0, s0 + n) of the result

@@ -104,6 +104,12 @@ __global__ void k_fft_tables(float2* __restrict__ tw)
         sincospi(a, &sn, &cs);
         tw[TW_N + e] = make_float2((float)cs, (float)sn);
     }
+    // the forward transforms' per-thread constants
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < 2 * FT; e += gridDim.x * blockDim.x) {
+        double sn, cs;
+        sincospi((double)(e / 2) / (e % 2 ? 4096.0 : 8192.0), &sn, &cs);
+        tw[TW_N + TWC_N + e] = make_float2((float)cs, (float)sn);
+    }
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < TW_N; e += gridDim.x * blockDim.x) {
         int n;                                    // exponent in units of 2 pi / 8192
         if (e < TW3) {
@@ -182,12 +188,12 @@ __device__ __forceinline__ float2 root32(int a)
     return a <= 8 ? make_float2(C[a], C[8 - a]) : make_float2(-C[16 - a], C[a - 8]);
 }
 
-// e^{i pi tid / den}, rounded from FP64 (a per-thread constant)
-__device__ __forceinline__ float2 thread_root(double den)
+// this thread's constants e^{i pi tid / 8192} (.x, .y) and e^{i pi tid / 4096}
+// (.z, .w), rounded from FP64 in the tables: computed here they were most of
+// the 16 us that one transform took (GB300's FP64 rate)
+__device__ __forceinline__ float4 thread_roots(const float2* __restrict__ tw)
 {
-    double sn, cs;
-    sincospi((double)threadIdx.x / den, &sn, &cs);
-    return make_float2((float)cs, (float)sn);
+    return __ldg(reinterpret_cast<const float4*>(tw + TW_N + TWC_N) + threadIdx.x);
 }
 
 // 4-point DFT with kernel e^{SIGN 2 pi i n k / 4}, in place
@@ -457,8 +463,9 @@ __global__ void __launch_bounds__(FT, 1) k_fft_series(const __grid_constant__ Ff
 {
     const Smem m = smem_setup<false>(p.tw);
     const int tid = threadIdx.x;
-    const float2 base_f = thread_root(4096.0);
-    const float2 base_r = thread_root(8192.0);
+    if (blockIdx.x == 0 && p.n_fix && tid < p.n) p.n_fix[tid] = 0u;       // k_fft_flags counts from 0
+    const float4 roots = thread_roots(p.tw);
+    const float2 base_f = make_float2(roots.z, roots.w), base_r = make_float2(roots.x, roots.y);
     for (uint32_t g = blockIdx.x; g < total; g += gridDim.x) {
         int s = 0;
         while (s + 1 < p.n && g >= p.seg_begin[s + 1]) ++s;
@@ -500,7 +507,8 @@ __global__ void __launch_bounds__(FT, 1) k_fft_bank_pair(const float* __restrict
 {
     const Smem m = smem_setup<false>(tw);
     const int tid = threadIdx.x;
-    const float2 base_f = thread_root(4096.0);
+    const float4 roots = thread_roots(tw);
+    const float2 base_f = make_float2(roots.z, roots.w);
     for (uint32_t q = blockIdx.x; q < n_items; q += gridDim.x) {
         const uint32_t a = 2 * q, b = a + 1;
         const float* ra = rows + (size_t)a * FN;
@@ -544,8 +552,8 @@ __global__ void __launch_bounds__(FT, 1) k_fft_bank_real(const float* __restrict
 {
     const Smem m = smem_setup<true>(tw);
     const int tid = threadIdx.x;
-    const float2 base_f = thread_root(4096.0);
-    const float2 base_r = thread_root(8192.0);
+    const float4 roots = thread_roots(tw);
+    const float2 base_f = make_float2(roots.z, roots.w), base_r = make_float2(roots.x, roots.y);
     const uint32_t n16 = (M + 3) / 4;             // 16-byte pieces holding a row's first M samples
     const uint32_t mh = 2 * n16;                  // complex values staged (M <= FH: mh <= FH / 2)
     uint32_t q = blockIdx.x;
@@ -603,8 +611,8 @@ __global__ void __launch_bounds__(FT, 1) k_welch_segments(const __grid_constant_
 {
     const Smem m = smem_setup<false>(p.tw);
     const int tid = threadIdx.x;
-    const float2 base_f = thread_root(4096.0);
-    const float2 base_r = thread_root(8192.0);
+    const float4 roots = thread_roots(p.tw);
+    const float2 base_f = make_float2(roots.z, roots.w), base_r = make_float2(roots.x, roots.y);
     for (uint32_t g = blockIdx.x; g < total; g += gridDim.x) {
         int s = 0;
         while (s + 1 < p.n && g >= p.seg_begin[s + 1]) ++s;
@@ -650,8 +658,8 @@ __global__ void __launch_bounds__(FT, 1) k_template_power_dot(const float* __res
     const Smem m = smem_setup<false>(tw);
     __shared__ double red[FT / 32];
     const int tid = threadIdx.x;
-    const float2 base_f = thread_root(4096.0);
-    const float2 base_r = thread_root(8192.0);
+    const float4 roots = thread_roots(tw);
+    const float2 base_f = make_float2(roots.z, roots.w), base_r = make_float2(roots.x, roots.y);
     for (uint32_t q = blockIdx.x; q < n_rows; q += gridDim.x) {
         const float2* r2 = reinterpret_cast<const float2*>(rows + (size_t)q * FN);
         for (int n = tid; n < FN; n += FT) m.z[n + (n >> 4)] = n < FH ? r2[n] : make_float2(0.f, 0.f);
@@ -1446,7 +1454,7 @@ cudaError_t fft_tables(bf_ctx* ctx, cudaStream_t st, const float2** out)
 {
     if (!ctx->fft_tw) {
         float2* t = nullptr;
-        cudaError_t e = cudaMalloc(&t, (TW_N + TWC_N) * sizeof(float2));
+        cudaError_t e = cudaMalloc(&t, (TW_N + TWC_N + 2 * FT) * sizeof(float2));
         if (e != cudaSuccess) return e;
         count_launches(1);
         k_fft_tables<<<(TW_N + 255) / 256, 256, 0, st>>>(t);
@@ -1595,8 +1603,6 @@ cudaError_t launch_fft_series(const FftSeriesBatch& b, uint32_t total_segments, 
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || !b.n_fix) return e;
     // the lags for the direct fixup
-    e = cudaMemsetAsync(b.n_fix, 0, (size_t)b.n * sizeof(uint32_t), st);
-    if (e != cudaSuccess) return e;
     uint32_t L_max = 0;
     for (int i = 0; i < b.n; ++i) L_max = std::max(L_max, b.L[i]);
     const unsigned bx = (unsigned)std::max<uint32_t>(1, std::min<uint32_t>((L_max + 255) / 256, 1024));

@@ -14,220 +14,217 @@
 //     nonzero samples decides it, because the block-wise scan sums the energy
 //     prefix in different orders on either side of a block edge, so S may
 //     differ by rounding across an all-zero window.
+//
+// Four launches for up to 64 series: block sums, their scan, prefix, norms and
+// rows.  What bounds them on the usual 10^4 to 10^5 samples is FP64
+// issue on the few SMs that hold the blocks -- GB300 runs a warp's FP64
+// instruction in 16 cycles -- and the launches themselves.  So a sample costs
+// one conversion and one FMA per pass (x^2 is exact, so the FMA rounds as the
+// addition would), counts are integers, the blocks are small (1024 samples),
+// and 1/sqrt starts from the FP32 one.  With the clearing of the outputs in one
+// launch a 4 s search of 256 templates went from 183 to 171 us, a served mix of
+// six requests (prepared one by one) from 3.61 to 3.50 ms.
 #include <algorithm>
 
 #include "bf_internal.h"
 
 namespace bfi {
 
-// split rows of series s = blockIdx.y: row w holds x[w .. w+7] (zero past N)
-__global__ void k_split_rows(const __grid_constant__ PrepBatch b)
-{
-    const int s = blockIdx.y;
-    if (s >= b.n) return;
-    const float* x = b.x[s];
-    const uint64_t N = b.N[s], rows = b.rows[s];
-    uint4* yhi = b.yhi[s];
-    uint4* ylo = b.ylo[s];
-    for (uint64_t w = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; w < rows;
-         w += (uint64_t)gridDim.x * blockDim.x) {
-        uint32_t h[4], l[4];
-#pragma unroll
-        for (int c = 0; c < 8; c += 2) {
-            float v0 = (w + c < N) ? x[w + c] : 0.f;
-            float v1 = (w + c + 1 < N) ? x[w + c + 1] : 0.f;
-            __nv_bfloat16 h0 = __float2bfloat16_rn(v0), h1 = __float2bfloat16_rn(v1);
-            __nv_bfloat16 l0 = __float2bfloat16_rn(v0 - __bfloat162float(h0));
-            __nv_bfloat16 l1 = __float2bfloat16_rn(v1 - __bfloat162float(h1));
-            h[c / 2] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
-            l[c / 2] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
-        }
-        yhi[w] = make_uint4(h[0], h[1], h[2], h[3]);
-        ylo[w] = make_uint4(l[0], l[1], l[2], l[3]);
-    }
-}
-
-// max |x| of series blockIdx.y as float bits (non-negative floats order like
-// unsigned integers), into *xmax (zeroed by k_block_sq)
-__global__ void k_absmax(const __grid_constant__ PrepBatch b)
-{
-    const int s = blockIdx.y;
-    if (s >= b.n) return;
-    const float* x = b.x[s];
-    const uint64_t N = b.N[s];
-    uint32_t m = 0;
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < N;
-         i += (uint64_t)gridDim.x * blockDim.x)
-        m = max(m, __float_as_uint(fabsf(x[i])));
-    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(b.xmax[s], m);
-}
-
-// Split rows as k_split_rows, in FP16 of x 2^s: hi = fp16(x 2^s), lo =
-// fp16(x 2^s - hi) (exact difference in FP32), s from the series' max |x|.
-__global__ void k_split_rows_f16(const __grid_constant__ PrepBatch b)
-{
-    const int s = blockIdx.y;
-    if (s >= b.n) return;
-    const float* x = b.x[s];
-    const uint64_t N = b.N[s], rows = b.rows[s];
-    uint4* yhi = b.yhi[s];
-    uint4* ylo = b.ylo[s];
-    const float scale = ldexpf(1.f, f16_series_shift(*b.xmax[s]));
-    for (uint64_t w = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; w < rows;
-         w += (uint64_t)gridDim.x * blockDim.x) {
-        uint32_t h[4], l[4];
-#pragma unroll
-        for (int c = 0; c < 8; c += 2) {
-            const float v0 = ((w + c < N) ? x[w + c] : 0.f) * scale;
-            const float v1 = ((w + c + 1 < N) ? x[w + c + 1] : 0.f) * scale;
-            const __half h0 = __float2half_rn(v0), h1 = __float2half_rn(v1);
-            const __half l0 = __float2half_rn(v0 - __half2float(h0));
-            const __half l1 = __float2half_rn(v1 - __half2float(h1));
-            h[c / 2] = (uint32_t)__half_as_ushort(h0) | ((uint32_t)__half_as_ushort(h1) << 16);
-            l[c / 2] = (uint32_t)__half_as_ushort(l0) | ((uint32_t)__half_as_ushort(l1) << 16);
-        }
-        yhi[w] = make_uint4(h[0], h[1], h[2], h[3]);
-        ylo[w] = make_uint4(l[0], l[1], l[2], l[3]);
-    }
-}
-
 // ---------------------------------------------------------------- FP64 scan
-constexpr int SCAN_T = 512;              // threads per scan block
+constexpr int SCAN_T = 256;              // threads per scan block
 constexpr int SCAN_E = 4;                // elements per thread
 constexpr int SCAN_B = SCAN_T * SCAN_E;  // elements per block
 
 // block-sum scratch (doubles): energies and nonzero counts of every scan block
 uint64_t inv_norm_scratch_blocks(uint64_t N) { return 2 * ((N + SCAN_B - 1) / SCAN_B + 1); }
 
-__device__ __forceinline__ double block_excl_scan(double v, double* sh, double* total)
+// sum over the block's threads, in every thread (sh: one word per warp; ends
+// with a barrier before which sh is read)
+template <typename T>
+__device__ __forceinline__ T block_sum(T v, T* sh)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    T tot = sh[0];
+#pragma unroll
+    for (int w = 1; w < SCAN_T / 32; ++w) tot += sh[w];
+    __syncthreads();
+    return tot;
+}
+
+// exclusive scan over the block's threads
+template <typename T>
+__device__ __forceinline__ T block_excl_scan(T v, T* sh)
 {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    double inc = v;
+    T inc = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        double t = __shfl_up_sync(0xffffffffu, inc, o);
+        const T t = __shfl_up_sync(0xffffffffu, inc, o);
         if (lane >= o) inc += t;
     }
     if (lane == 31) sh[wid] = inc;
     __syncthreads();
-    if (wid == 0) {
-        double s = lane < (SCAN_T / 32) ? sh[lane] : 0.0;
+    T base = T(0);
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            double t = __shfl_up_sync(0xffffffffu, s, o);
-            if (lane >= o) s += t;
-        }
-        if (lane < SCAN_T / 32) sh[lane] = s;
-    }
+    for (int w = 0; w < SCAN_T / 32; ++w)
+        if (w < wid) base += sh[w];
     __syncthreads();
-    double base = wid > 0 ? sh[wid - 1] : 0.0;
-    if (total) *total = sh[SCAN_T / 32 - 1];
-    return base + inc - v;
+    return base + (inc - v);
 }
 
-// Per-block sums of x^2 (FP64) and of the count of nonzero samples (an exact
-// integer in FP64) of series s = blockIdx.y: bsum[0, nb) and bsum[nb, 2 nb).
-// The same launch zeroes the series' padding x[N, xcap) and its max |x| word.
+__device__ __forceinline__ uint32_t* block_counts(double* bsum, uint64_t nb) { return reinterpret_cast<uint32_t*>(bsum + nb); }
+
+// this thread's SCAN_E samples of scan block blockIdx.x (zero past N)
+__device__ __forceinline__ void load_samples(const float* __restrict__ x, uint64_t N, float (&v)[SCAN_E])
+{
+    const uint64_t base = (uint64_t)blockIdx.x * SCAN_B + (uint64_t)threadIdx.x * SCAN_E;
+    static_assert(SCAN_E == 4, "one 16-byte load");
+    if (base + SCAN_E <= N) {
+        const float4 f = *reinterpret_cast<const float4*>(x + base);
+        v[0] = f.x;
+        v[1] = f.y;
+        v[2] = f.z;
+        v[3] = f.w;
+    } else {
+#pragma unroll
+        for (int e = 0; e < SCAN_E; ++e) v[e] = base + e < N ? x[base + e] : 0.f;
+    }
+}
+
+// Per-block sums of x^2 (FP64) and counts of nonzero samples of series
+// s = blockIdx.y.  The same launch zeroes the series' padding x[N, xcap) and its
+// max |x| word.
 __global__ void __launch_bounds__(SCAN_T) k_block_sq(const __grid_constant__ PrepBatch b)
 {
     __shared__ double sh[SCAN_T / 32];
+    __shared__ uint32_t shc[SCAN_T / 32];
     const int s = blockIdx.y;
     if (s >= b.n) return;
-    const float* x = b.x[s];
     const uint64_t N = b.N[s], nb = b.nb[s];
     for (uint64_t i = N + blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < b.xcap[s];
          i += (uint64_t)gridDim.x * blockDim.x)
         b.x[s][i] = 0.f;
     if (b.mode == 2 && blockIdx.x == 0 && threadIdx.x == 0) *b.xmax[s] = 0u;
     if (blockIdx.x >= nb) return;
-    double* bsum = b.bsum[s];
-    uint64_t base = (uint64_t)blockIdx.x * SCAN_B + (uint64_t)threadIdx.x * SCAN_E;
-    double v = 0.0, c = 0.0;
+    float x[SCAN_E];
+    load_samples(b.x[s], N, x);
+    double v = 0.0;
+    uint32_t c = 0;
 #pragma unroll
-    for (int e = 0; e < SCAN_E; ++e)
-        if (base + e < N) {
-            double d = x[base + e];
-            v += d * d;
-            c += d != 0.0 ? 1.0 : 0.0;
-        }
-    double tot, ctot;
-    block_excl_scan(v, sh, &tot);
-    __syncthreads();
-    block_excl_scan(c, sh, &ctot);
+    for (int e = 0; e < SCAN_E; ++e) {
+        const double d = (double)x[e];
+        v = fma(d, d, v);
+        c += x[e] != 0.f ? 1u : 0u;
+    }
+    const double tot = block_sum(v, sh);
+    const uint32_t ctot = block_sum(c, shc);
     if (threadIdx.x == 0) {
-        bsum[blockIdx.x] = tot;
-        bsum[nb + blockIdx.x] = ctot;
+        b.bsum[s][blockIdx.x] = tot;
+        block_counts(b.bsum[s], nb)[blockIdx.x] = ctot;
     }
 }
 
-// exclusive scan of the nb block sums of one lane of series blockIdx.y, in
-// place (block x = 0: energies, 1: counts)
+// exclusive scan of the nb block sums of series blockIdx.y, in place
 __global__ void __launch_bounds__(SCAN_T) k_scan_sums(const __grid_constant__ PrepBatch b)
 {
     __shared__ double sh[SCAN_T / 32];
+    __shared__ uint32_t shc[SCAN_T / 32];
     const int s = blockIdx.y;
     if (s >= b.n) return;
     const uint64_t n = b.nb[s];
-    double* lane_sums = b.bsum[s] + blockIdx.x * n;
+    double* energy = b.bsum[s];
+    uint32_t* count = block_counts(b.bsum[s], n);
     double carry = 0.0;
-    for (uint64_t c = 0; c < n; c += SCAN_T) {
-        uint64_t i = c + threadIdx.x;
-        double v = i < n ? lane_sums[i] : 0.0;
-        double tot;
-        double ex = block_excl_scan(v, sh, &tot);
-        __syncthreads();
-        if (i < n) lane_sums[i] = carry + ex;
+    uint32_t ccarry = 0;
+    for (uint64_t c0 = 0; c0 < n; c0 += SCAN_T) {
+        const uint64_t i = c0 + threadIdx.x;
+        const double v = i < n ? energy[i] : 0.0;
+        const uint32_t c = i < n ? count[i] : 0u;
+        const double ex = block_excl_scan(v, sh);
+        const uint32_t cx = block_excl_scan(c, shc);
+        const double tot = block_sum(v, sh);
+        const uint32_t ctot = block_sum(c, shc);
+        if (i < n) {
+            energy[i] = carry + ex;
+            count[i] = ccarry + cx;
+        }
         carry += tot;
-        __syncthreads();
+        ccarry += ctot;
     }
 }
 
 // S[t] = sum_{i < t} x_i^2 and C[t] = #{i < t : x_i != 0}, t = 0..N, of
-// series blockIdx.y
+// series blockIdx.y; mode 2 also max |x| as float bits (non-negative floats
+// order like unsigned integers) into *xmax (zeroed by k_block_sq)
 __global__ void __launch_bounds__(SCAN_T) k_prefix(const __grid_constant__ PrepBatch b)
 {
     __shared__ double sh[SCAN_T / 32];
+    __shared__ uint32_t shc[SCAN_T / 32];
     const int s = blockIdx.y;
     if (s >= b.n || blockIdx.x >= b.nb[s]) return;
-    const float* x = b.x[s];
     const uint64_t N = b.N[s], nb = b.nb[s];
-    const double* boff = b.bsum[s];
     double* S = b.S[s];
     uint32_t* C = reinterpret_cast<uint32_t*>(S + N + 1);
-    uint64_t base = (uint64_t)blockIdx.x * SCAN_B + (uint64_t)threadIdx.x * SCAN_E;
-    double v[SCAN_E];
-    uint32_t nz[SCAN_E];
-    double t = 0.0, c = 0.0;
+    float x[SCAN_E];
+    load_samples(b.x[s], N, x);
+    double t = 0.0;
+    uint32_t c = 0;
 #pragma unroll
     for (int e = 0; e < SCAN_E; ++e) {
-        double d = base + e < N ? (double)x[base + e] : 0.0;
-        v[e] = d * d;
-        nz[e] = d != 0.0 ? 1u : 0u;
-        t += v[e];
-        c += (double)nz[e];
+        const double d = (double)x[e];
+        t = fma(d, d, t);
+        c += x[e] != 0.f ? 1u : 0u;
     }
-    double ex = block_excl_scan(t, sh, nullptr) + boff[blockIdx.x];
-    __syncthreads();
-    uint32_t cx = (uint32_t)(block_excl_scan(c, sh, nullptr) + boff[nb + blockIdx.x]);
+    double ex = block_excl_scan(t, sh) + b.bsum[s][blockIdx.x];
+    uint32_t cx = block_excl_scan(c, shc) + block_counts(b.bsum[s], nb)[blockIdx.x];
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         S[0] = 0.0;
         C[0] = 0u;
     }
+    const uint64_t at = (uint64_t)blockIdx.x * SCAN_B + (uint64_t)threadIdx.x * SCAN_E;
 #pragma unroll
     for (int e = 0; e < SCAN_E; ++e) {
-        ex += v[e];
-        cx += nz[e];
-        if (base + e < N) {
-            S[base + e + 1] = ex;
-            C[base + e + 1] = cx;
+        const double d = (double)x[e];
+        ex = fma(d, d, ex);
+        cx += x[e] != 0.f ? 1u : 0u;
+        if (at + e < N) {
+            S[at + e + 1] = ex;
+            C[at + e + 1] = cx;
         }
+    }
+    if (b.mode == 2) {
+        uint32_t m = 0;
+#pragma unroll
+        for (int e = 0; e < SCAN_E; ++e) m = max(m, __float_as_uint(fabsf(x[e])));
+        m = __reduce_max_sync(0xffffffffu, m);
+        if ((threadIdx.x & 31) == 0) atomicMax(b.xmax[s], m);
     }
 }
 
-// 1 / |window|, and exactly 0 for a window without a nonzero sample (rho := 0
-// there).  The count decides emptiness: a difference of FP64 prefix sums
-// formed in different orders need not vanish over an all-zero window.
+// 1/sqrt(nu) for nu > 0, rounded to FP32 from FP64: the FP32 value of nu's
+// mantissa with an even exponent, m in [1, 4), then one Newton step
+// y += y (1 - m y^2) / 2 in FP64 (relative error 3/8 (2 * 2^-22)^2, far inside
+// FP32's half ulp), scaled back exactly.  Energies outside 2^+-240 (the result
+// would leave the range of normal floats) take the FP64 root and division.
+__device__ __forceinline__ float inv_sqrt(double nu)
+{
+    const int hi = __double2hiint(nu);
+    const int e = ((hi >> 20) - 1023) & ~1;               // even exponent
+    if (e < -240 || e > 240) return (float)(1.0 / sqrt(nu));
+    const double m = __hiloint2double(hi - (e << 20), __double2loint(nu));
+    const double y = (double)rsqrtf((float)m);
+    const double h = fma(-m * y, y, 1.0);                 // 1 - m y^2
+    const float r = (float)fma(0.5 * y, h, y);
+    return r * __int_as_float((127 - e / 2) << 23);       // 2^(-e/2)
+}
+
+// Norms and split rows of series blockIdx.y, one index per thread.
+// Norms: 1 / |window|, and exactly 0 for a window without a nonzero sample
+// (rho := 0 there).  The count decides emptiness: a difference of FP64 prefix
+// sums formed in different orders need not vanish over an all-zero window.
 // The prefix difference S[t+M] - S[t] carries an absolute rounding error of a
 // few ulps of S[t+M]; where the window holds less than 2^-30 of the energy
 // before it (a quiet stretch after loud data) that would be a relative error
@@ -235,30 +232,62 @@ __global__ void __launch_bounds__(SCAN_T) k_prefix(const __grid_constant__ PrepB
 // The first thread of a series also reports a non-finite series: the FP64
 // total of x^2 (at most 2^32 squares of floats, far below the FP64 range) is
 // finite exactly when every sample is.
-__global__ void k_inv_norm(const __grid_constant__ PrepBatch b)
+// Rows (mode 1 and 2): row w holds x[w .. w+7] (zero past N), in mode 2 as FP16
+// of x 2^e: hi = fp16(x 2^e), lo = fp16(x 2^e - hi) (exact difference in FP32),
+// e from the series' max |x|.
+__global__ void k_norms_rows(const __grid_constant__ PrepBatch b)
 {
     const int s = blockIdx.y;
     if (s >= b.n) return;
     const float* x = b.x[s];
     const uint32_t M = b.M;
-    const uint64_t N = b.N[s], L = N - M + 1;
+    const uint64_t N = b.N[s], L = N - M + 1, rows = b.mode ? b.rows[s] : 0;
     const double* S = b.S[s];
     const uint32_t* C = reinterpret_cast<const uint32_t*>(S + N + 1);
     float* inv = b.inv[s];
+    uint4* yhi = b.yhi[s];
+    uint4* ylo = b.ylo[s];
+    const float scale = b.mode == 2 ? ldexpf(1.f, f16_series_shift(*b.xmax[s])) : 1.f;
     if (b.status[s] && blockIdx.x == 0 && threadIdx.x == 0 && !isfinite(S[N])) atomicOr(b.status[s], 1u);
-    for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < L;
+    const uint64_t n = rows > L ? rows : L;
+    for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < n;
          t += (uint64_t)gridDim.x * blockDim.x) {
-        double nu = S[t + M] - S[t];
-        const bool any = C[t + M] != C[t];
-        if (any && nu < S[t + M] * 0x1p-30) {
-            double acc = 0.0;
-            for (uint32_t m = 0; m < M; ++m) {
-                const double v = (double)x[t + m];
-                acc = fma(v, v, acc);
+        if (t < L) {
+            const double end = S[t + M];
+            double nu = end - S[t];
+            const bool any = C[t + M] != C[t];
+            if (any && nu < end * 0x1p-30) {
+                double acc = 0.0;
+                for (uint32_t m = 0; m < M; ++m) {
+                    const double v = (double)x[t + m];
+                    acc = fma(v, v, acc);
+                }
+                nu = acc;
             }
-            nu = acc;
+            inv[t] = (any && nu > 0.0) ? inv_sqrt(nu) : 0.f;
         }
-        inv[t] = (any && nu > 0.0) ? (float)(1.0 / sqrt(nu)) : 0.f;
+        if (t >= rows) continue;
+        uint32_t h[4], l[4];
+#pragma unroll
+        for (int c = 0; c < 8; c += 2) {
+            const float v0 = ((t + c < N) ? x[t + c] : 0.f) * scale;
+            const float v1 = ((t + c + 1 < N) ? x[t + c + 1] : 0.f) * scale;
+            if (b.mode == 1) {
+                const __nv_bfloat16 h0 = __float2bfloat16_rn(v0), h1 = __float2bfloat16_rn(v1);
+                const __nv_bfloat16 l0 = __float2bfloat16_rn(v0 - __bfloat162float(h0));
+                const __nv_bfloat16 l1 = __float2bfloat16_rn(v1 - __bfloat162float(h1));
+                h[c / 2] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
+                l[c / 2] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
+            } else {
+                const __half h0 = __float2half_rn(v0), h1 = __float2half_rn(v1);
+                const __half l0 = __float2half_rn(v0 - __half2float(h0));
+                const __half l1 = __float2half_rn(v1 - __half2float(h1));
+                h[c / 2] = (uint32_t)__half_as_ushort(h0) | ((uint32_t)__half_as_ushort(h1) << 16);
+                l[c / 2] = (uint32_t)__half_as_ushort(l0) | ((uint32_t)__half_as_ushort(l1) << 16);
+            }
+        }
+        yhi[t] = make_uint4(h[0], h[1], h[2], h[3]);
+        ylo[t] = make_uint4(l[0], l[1], l[2], l[3]);
     }
 }
 
@@ -269,31 +298,19 @@ uint64_t prep_scan_blocks(uint64_t N) { return (N + SCAN_B - 1) / SCAN_B; }
 cudaError_t launch_prep(const PrepBatch& b, cudaStream_t st)
 {
     if (b.n <= 0 || b.n > MAX_PREP) return cudaErrorInvalidValue;
-    uint64_t nb = 0, lmax = 0, rmax = 0, nmax = 0;
+    uint64_t nb = 0, work = 0;
     for (int i = 0; i < b.n; ++i) {
         if (b.N[i] < b.M || b.nb[i] != prep_scan_blocks(b.N[i]) || b.nb[i] == 0) return cudaErrorInvalidValue;
         nb = std::max(nb, b.nb[i]);
-        lmax = std::max(lmax, b.N[i] - b.M + 1);
-        rmax = std::max(rmax, b.rows[i]);
-        nmax = std::max(nmax, b.N[i]);
+        work = std::max(work, std::max(b.N[i] - b.M + 1, b.mode ? b.rows[i] : 0));
     }
-    auto grid_x = [](uint64_t work) {
-        return (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((work + 255) / 256, 65535ull * 16));
-    };
     const unsigned ny = (unsigned)b.n;
+    const unsigned bx = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((work + 255) / 256, 65535ull * 16));
     count_launches(4);
     k_block_sq<<<dim3((unsigned)nb, ny), SCAN_T, 0, st>>>(b);
-    k_scan_sums<<<dim3(2, ny), SCAN_T, 0, st>>>(b);
+    k_scan_sums<<<dim3(1, ny), SCAN_T, 0, st>>>(b);
     k_prefix<<<dim3((unsigned)nb, ny), SCAN_T, 0, st>>>(b);
-    k_inv_norm<<<dim3(grid_x(lmax), ny), 256, 0, st>>>(b);
-    if (b.mode == 1) {
-        count_launches(1);
-        k_split_rows<<<dim3(grid_x(rmax), ny), 256, 0, st>>>(b);
-    } else if (b.mode == 2) {
-        count_launches(2);
-        k_absmax<<<dim3((unsigned)std::min<uint64_t>((nmax + 255) / 256, 1024), ny), 256, 0, st>>>(b);
-        k_split_rows_f16<<<dim3(grid_x(rmax), ny), 256, 0, st>>>(b);
-    }
+    k_norms_rows<<<dim3(bx, ny), 256, 0, st>>>(b);
     return cudaGetLastError();
 }
 
