@@ -111,6 +111,50 @@ bool Allocator::fits(size_t bytes) const
     return live_ + round_alloc(bytes) <= budget_;
 }
 
+// ---------------------------------------------------------------- page-locked host memory
+HostPool::~HostPool()
+{
+    for (auto& kv : size_of_) cudaFreeHost(kv.first);
+}
+
+void* HostPool::alloc(size_t bytes)
+{
+    size_t b = 4096;
+    while (b < bytes) b <<= 1;
+    std::lock_guard<std::mutex> g(mu_);
+    auto it = cache_.find(b);
+    if (it != cache_.end()) {
+        void* p = it->second;
+        cache_.erase(it);
+        return p;
+    }
+    if (held_ + b > cap_) {
+        for (auto& kv : cache_) {                       // give back cached blocks of other sizes
+            cudaFreeHost(kv.second);
+            held_ -= kv.first;
+            size_of_.erase(kv.second);
+        }
+        cache_.clear();
+        if (held_ + b > cap_) return nullptr;
+    }
+    void* p = nullptr;
+    if (cudaHostAlloc(&p, b, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    held_ += b;
+    size_of_[p] = b;
+    return p;
+}
+
+void HostPool::release(void* p)
+{
+    if (!p) return;
+    std::lock_guard<std::mutex> g(mu_);
+    auto it = size_of_.find(p);
+    if (it != size_of_.end()) cache_.emplace(it->second, p);
+}
+
 // ---------------------------------------------------------------- helpers
 bool is_device_ptr(const void* p)
 {
@@ -451,6 +495,9 @@ static void free_result_buffers(bf_result* r)
                     (void*)r->cand, (void*)r->cand_count, (void*)r->sigma_pred})
         mem.release(p);
     r->sigma_pred = nullptr;
+    r->ctx->host_mem->release(r->host);
+    r->host = nullptr;
+    r->host_ready = false;
     r->canaries.clear();
     for (void* p : r->scratch) mem.release(p);
     r->scratch.clear();
@@ -528,10 +575,14 @@ bf_status resolve_opts(const bf_bank* bank, const bf_opts* in, bf_opts* o)
     return BF_OK;
 }
 
+// Largest host copy of a result: a search of 65,536 templates in four series
+// (3.2 MB).  Larger ones are copied when asked for, at the link's full rate.
+constexpr size_t HOST_COPY_BYTES = size_t(4) << 20;
+
 // Allocates and zeroes the outputs of a result for series of the given lengths.
 bf_status alloc_result(bf_ctx* ctx, const bf_bank* bank, const bf_opts& o,
                        const std::vector<size_t>& lengths, double fs, cudaStream_t st,
-                       bf_result** out)
+                       bool host_copy, bf_result** out)
 {
     std::unique_ptr<bf_result> r(new bf_result());
     r->ctx = ctx;
@@ -611,6 +662,13 @@ bf_status alloc_result(bf_ctx* ctx, const bf_bank* bank, const bf_opts& o,
         return BF_ENOMEM;
     }
     r->map_total = map_total;
+    if (host_copy) {
+        // up to HOST_COPY_BYTES the outputs too, beyond them the head only
+        const size_t data = 64 + (S * K * 3 + K + (r->hist ? S * r->nbins : 0)) * 4;
+        r->host_data = data <= HOST_COPY_BYTES;
+        r->host = static_cast<HostHead*>(ctx->host_mem->alloc(r->host_data ? data : sizeof(HostHead)));
+        if (!r->host) r->host_data = false;
+    }
     cudaError_t e = cudaSuccess;
     for (unsigned char* c : r->canaries)
         if (e == cudaSuccess) e = cudaMemsetAsync(c, CANARY_FILL, CANARY_BYTES, st);
@@ -678,13 +736,36 @@ bf_status finalize_result(bf_ctx* ctx, const bf_bank* bank, bf_result* r, cudaSt
             f.map = r->map ? r->map + r->map_off[s] : nullptr;
             f.L = (uint32_t)(r->lengths[s] - bank->M + 1);
             f.nt = r->map_nt[s];
+            if (r->host_data) {
+                f.h_vmax = r->host_vmax() + s * K;
+                f.h_argmax = r->host_argmax() + s * K;
+                f.h_sigma = r->host_sigma() + s * K;
+            }
         }
         e = launch_finalize(fp, (uint32_t)K, r->nbins, st);
         if (e == cudaSuccess && r->map)
             e = launch_paint(r->cand, r->cand_count, r->cand_cap, bank->d_params, fp, bank->M,
                              r->fs, r->dt, r->df, r->map_nf, (unsigned)ctx->n_sm, st);
     }
-    if (e == cudaSuccess) e = launch_mean_max(r->vmax, (uint32_t)S, (uint32_t)K, r->mean_max, st);
+    if (e == cudaSuccess) {
+        PublishParams p{};
+        p.vmax = r->vmax;
+        p.mean = r->mean_max;
+        p.n_series = (uint32_t)S;
+        p.K = (uint32_t)K;
+        p.head = r->host;
+        p.err = ctx->d_err;
+        p.counts = r->cand_count;
+        if (r->host_data) {
+            p.h_mean = r->host_mean();
+            if (r->hist) {
+                p.hist = r->hist;
+                p.h_hist = r->host_hist();
+                p.n_hist = (uint64_t)S * r->nbins;
+            }
+        }
+        e = launch_publish(p, st);
+    }
     if (e != cudaSuccess) return cuda_fail(e, "finalize");
     return BF_OK;
 }
@@ -846,11 +927,8 @@ bf_status check_canaries(const bf_result* r)
     return BF_OK;
 }
 
-bf_status result_status(const bf_result* r)
+static bf_status status_of(unsigned int w)
 {
-    unsigned int w = 0;
-    cudaError_t e = cudaMemcpy(&w, r->status, sizeof w, cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(e, "reading the result status");
     if (w & 1u) {
         set_error("a series holds a non-finite sample (NaN or infinity)");
         return BF_EINVAL;
@@ -858,17 +936,49 @@ bf_status result_status(const bf_result* r)
     return BF_OK;
 }
 
-bf_status check_device_status(bf_ctx* ctx)
+static bf_status device_status_of(bf_ctx* ctx, int h)
 {
-    int h = 0;
-    cudaError_t e = cudaMemcpy(&h, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(e, "reading kernel status");
     if (h != DEV_OK) {
         cudaMemset(ctx->d_err, 0, sizeof(int));
         if (h == DEV_BOUNDS) set_error("a kernel's bounds check failed (debug build)");
         else set_error("kernel reported internal timeout (code %d)", h);
         return BF_EDEVICE;
     }
+    return BF_OK;
+}
+
+bf_status result_status(const bf_result* r)
+{
+    unsigned int w = 0;
+    cudaError_t e = cudaMemcpy(&w, r->status, sizeof w, cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) return cuda_fail(e, "reading the result status");
+    return status_of(w);
+}
+
+bf_status check_device_status(bf_ctx* ctx)
+{
+    int h = 0;
+    cudaError_t e = cudaMemcpy(&h, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) return cuda_fail(e, "reading kernel status");
+    return device_status_of(ctx, h);
+}
+
+bf_status result_complete(bf_result* r)
+{
+    HostHead h{};
+    if (r->host) {
+        h = *r->host;
+    } else {
+        cudaError_t e = cudaMemcpy(&h.err, r->ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost);
+        if (e == cudaSuccess) e = cudaMemcpy(&h.cand_count, r->cand_count, 2 * sizeof(unsigned int), cudaMemcpyDeviceToHost);
+        if (e != cudaSuccess) return cuda_fail(e, "reading the search's status");
+    }
+    bf_status st = device_status_of(r->ctx, h.err);
+    if (st == BF_OK) st = check_canaries(r);        // debug builds: no output written past its end
+    if (st == BF_OK) st = status_of(h.status);      // every sample must be finite
+    if (st != BF_OK) return st;
+    r->n_candidates = h.cand_count;
+    r->host_ready = r->host != nullptr;
     return BF_OK;
 }
 
@@ -1095,8 +1205,11 @@ bf_status bf_init(const bf_config* cfg, bf_ctx** out)
     ctx->n_sm = prop.multiProcessorCount;
     ctx->cfg = c;
     ctx->mem.reset(new Allocator(c.hbm_budget));
+    ctx->host_mem.reset(new HostPool(size_t(64) << 20));
     e = cudaStreamCreateWithFlags(&ctx->stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&ctx->aux, cudaStreamNonBlocking);
+    for (cudaEvent_t& ev : ctx->ev)
+        if (e == cudaSuccess) e = cudaEventCreate(&ev);
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamCreate");
     e = cudaMalloc(&ctx->d_err, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(ctx->d_err, 0, sizeof(int));
@@ -1124,6 +1237,9 @@ void bf_destroy(bf_ctx* ctx)
     serve_shutdown(ctx);
     cudaStreamSynchronize(ctx->stream);
     ctx->mem.reset();
+    ctx->host_mem.reset();
+    for (cudaEvent_t ev : ctx->ev)
+        if (ev) cudaEventDestroy(ev);
     cudaFree(ctx->d_err);
     if (ctx->fft_tw) cudaFree(ctx->fft_tw);
     cudaStreamDestroy(ctx->stream);
@@ -1380,7 +1496,7 @@ bf_status bf_correlate(bf_ctx* ctx, const bf_bank* bank, const float* const* ser
 
     std::vector<size_t> lens(lengths, lengths + n_series);
     bf_result* r = nullptr;
-    st = alloc_result(ctx, bank, o, lens, fs, strm, &r);
+    st = alloc_result(ctx, bank, o, lens, fs, strm, sync, &r);
     if (st) return st;
     std::unique_ptr<bf_result, void (*)(bf_result*)> guard(r, bf_result_destroy);
 
@@ -1445,12 +1561,7 @@ bf_status bf_correlate(bf_ctx* ctx, const bf_bank* bank, const float* const* ser
         if (st) return st;
     }
 
-    cudaEvent_t e0 = nullptr, e1 = nullptr;
-    if (sync) {
-        cudaEventCreate(&e0);
-        cudaEventCreate(&e1);
-        cudaEventRecord(e0, strm);
-    }
+    if (sync) cudaEventRecord(ctx->ev[0], strm);
     // lags per tile: fixed by the caller, else the autotuner's choice (for a
     // generated bank it is made on the first synthesised chunk)
     int lt = o.precision == BF_FP32 ? SIMT_TILE_L : fft ? 0 : o.tile_lags;
@@ -1461,34 +1572,20 @@ bf_status bf_correlate(bf_ctx* ctx, const bf_bank* bank, const float* const* ser
                         ? gen_launch(ctx, bank, o, segs, r, strm, lt, ring)
                         : launch_segments(ctx, segs, o.precision, r->thr, r->cand, r->cand_count,
                                           r->cand_cap, strm, nullptr, lt);
-    if (sync) cudaEventRecord(e1, strm);
-    if (e != cudaSuccess) {
-        if (e0) { cudaEventDestroy(e0); cudaEventDestroy(e1); }
-        return cuda_fail(e, "correlation launch");
-    }
+    if (sync) cudaEventRecord(ctx->ev[1], strm);
+    if (e != cudaSuccess) return cuda_fail(e, "correlation launch");
     {
         NvtxRange fr("finalize");
         st = finalize_result(ctx, bank, r, strm);
     }
-    if (st) {
-        if (e0) { cudaEventDestroy(e0); cudaEventDestroy(e1); }
-        return st;
-    }
+    if (st) return st;
     if (sync) {
         e = cudaStreamSynchronize(strm);
         float ms = 0.f;
-        cudaEventElapsedTime(&ms, e0, e1);
+        cudaEventElapsedTime(&ms, ctx->ev[0], ctx->ev[1]);
         r->kernel_ms = ms;
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
         if (e != cudaSuccess) return cuda_fail(e, "correlation");
-        st = check_device_status(ctx);
-        if (st) return st;
-        // debug builds: no output written past its end
-        st = check_canaries(r);
-        if (st) return st;
-        // every sample must be finite (the series preparation flags it)
-        st = result_status(r);
+        st = result_complete(r);
         for (size_t s = 0; st == BF_EINVAL && s < n_series; ++s) {
             // name the series: the one whose FP64 total of x^2 is not finite
             double total = 0.0;
@@ -1499,9 +1596,6 @@ bf_status bf_correlate(bf_ctx* ctx, const bf_bank* bank, const float* const* ser
             }
         }
         if (st) return st;
-        unsigned int cnt = 0;
-        cudaMemcpy(&cnt, r->cand_count, sizeof cnt, cudaMemcpyDeviceToHost);
-        r->n_candidates = cnt;
         for (void* p : r->scratch) ctx->mem->release(p);
         r->scratch.clear();
     }
@@ -1528,7 +1622,7 @@ bf_status bf_result_info_get(const bf_result* r, bf_result_info* info)
     info->correlations = r->correlations;
     info->useful_flops = 2.0 * r->M * r->correlations;
     uint64_t n = r->n_candidates;
-    if (r->cand_count && n == 0) {
+    if (r->cand_count && n == 0 && !r->host_ready) {
         unsigned int c = 0;
         if (cudaMemcpy(&c, r->cand_count, sizeof c, cudaMemcpyDeviceToHost) == cudaSuccess) n = c;
     }
@@ -1592,6 +1686,18 @@ static bf_status copy_series(const bf_result* r, size_t s, float* vmax, int32_t*
     const size_t K = r->K;
     const cudaMemcpyKind d2h = cudaMemcpyDeviceToHost;
     cudaError_t e = cudaSuccess;
+    if (!async && r->host_ready && r->host_data) {
+        // complete, and in host memory already
+        if (vmax) memcpy(vmax, r->host_vmax() + s * K, K * 4);
+        if (argmax) memcpy(argmax, r->host_argmax() + s * K, K * 4);
+        if (sigma) memcpy(sigma, r->host_sigma() + s * K, K * 4);
+        if (hist) memcpy(hist, r->host_hist() + s * r->nbins, r->nbins * 4);
+        if (!map) return BF_OK;
+        vmax = nullptr;
+        argmax = nullptr;
+        sigma = nullptr;
+        hist = nullptr;
+    }
     if (vmax) e = cudaMemcpyAsync(vmax, r->vmax + s * K, K * 4, d2h, st);
     if (e == cudaSuccess && argmax) e = cudaMemcpyAsync(argmax, r->argmax + s * K, K * 4, d2h, st);
     if (e == cudaSuccess && sigma) e = cudaMemcpyAsync(sigma, r->sigma + s * K, K * 4, d2h, st);
@@ -1657,6 +1763,10 @@ bf_status bf_result_copy_map_cells_async(const bf_result* r, size_t s, uint32_t*
 bf_status bf_result_copy_mean_max(const bf_result* r, float* out)
 {
     if (!r || !out) { set_error("NULL argument"); return BF_EINVAL; }
+    if (r->host_ready && r->host_data) {
+        memcpy(out, r->host_mean(), r->K * 4);
+        return BF_OK;
+    }
     cudaSetDevice(r->ctx->device);
     cudaError_t e = cudaMemcpy(out, r->mean_max, r->K * 4, cudaMemcpyDeviceToHost);
     return e == cudaSuccess ? BF_OK : cuda_fail(e, "result copy");
@@ -1741,7 +1851,7 @@ bf_status bf_result_copy_sigma_pred(const bf_result* r, size_t s, float* host)
 static size_t kept_tails(const bf_result* r)
 {
     uint64_t n = r->n_candidates;
-    if (r->cand_count) {
+    if (r->cand_count && !r->host_ready) {
         unsigned int c = 0;
         if (cudaMemcpy(&c, r->cand_count, sizeof c, cudaMemcpyDeviceToHost) == cudaSuccess) n = c;
     }

@@ -312,6 +312,30 @@ struct FinalizeSeries {
     float* map;
     uint32_t L;
     uint32_t nt;
+    // the result's host copy (mapped page-locked memory), or nullptr
+    float* h_vmax;
+    int32_t* h_argmax;
+    float* h_sigma;
+};
+// What the last kernel of a search writes for the host: the per-template mean,
+// and into the result's host copy (mapped page-locked memory; head may be
+// nullptr) the status words, the mean and the histograms.
+struct HostHead {
+    int err;                        // the context's status word
+    unsigned int cand_count;
+    unsigned int status;            // bit 0: a series holds a non-finite sample
+};
+struct PublishParams {
+    const float* vmax;              // [n_series][K]
+    float* mean;
+    uint32_t n_series, K;
+    HostHead* head;
+    const int* err;
+    const unsigned int* counts;     // cand_count, status
+    float* h_mean;                  // nullptr: only the head
+    const uint32_t* hist;           // n_hist words, or nullptr
+    uint32_t* h_hist;
+    uint64_t n_hist;
 };
 // arrays of 32-bit words, 16-byte aligned, zeroed by one launch
 struct ClearParams {
@@ -364,8 +388,7 @@ cudaError_t launch_coincidence(const float* A, const float* B, uint32_t nt, uint
                                uint32_t dt, unsigned int* out, int n_sm, cudaStream_t s);
 cudaError_t launch_skewnorm_fit(const float* v, uint64_t n, double* acc, double* out, int n_sm,
                                 cudaStream_t s);
-cudaError_t launch_mean_max(const float* vmax, uint32_t n_series, uint32_t K, float* mean,
-                            cudaStream_t s);
+cudaError_t launch_publish(const PublishParams& p, cudaStream_t s);
 cudaError_t launch_paint(const Candidate* cand, const unsigned int* count,
                          unsigned int cap, const ChirpDev* params,
                          const FinalizeParams& p, uint32_t M, double fs, double dt,
@@ -404,6 +427,23 @@ struct Allocator {
     mutable std::mutex mu_;
 };
 
+// Page-locked host memory, mapped into the device's address space, for the host
+// copies of results: blocks of powers of two from 4 KiB, kept for reuse, at most
+// `cap` bytes in all (alloc then returns nullptr, and the results are copied
+// when asked for instead).  Thread-safe.
+struct HostPool {
+    explicit HostPool(size_t cap) : cap_(cap) {}
+    ~HostPool();
+    void* alloc(size_t bytes);
+    void release(void* p);
+
+  private:
+    size_t cap_, held_ = 0;
+    std::multimap<size_t, void*> cache_;
+    std::unordered_map<void*, size_t> size_of_;
+    std::mutex mu_;
+};
+
 struct ServeState;
 
 }  // namespace bfi
@@ -415,6 +455,8 @@ struct bf_ctx {
     cudaStream_t stream = nullptr;
     cudaStream_t aux = nullptr;         // template synthesis of generated banks
     std::unique_ptr<bfi::Allocator> mem;
+    std::unique_ptr<bfi::HostPool> host_mem;
+    cudaEvent_t ev[2] = {nullptr, nullptr};   // kernel time of synchronous calls (under launch_mu)
     int* d_err = nullptr;               // kernel status word
     std::mutex launch_mu;               // serialises use of d_err / stream
     bfi::ServeState* serve = nullptr;   // owned; freed by serve_shutdown
@@ -473,6 +515,16 @@ struct bf_result {
     // device word after cand_count, zeroed with it: bit 0 is set by the series
     // preparation when a series holds a non-finite sample
     unsigned int* status = nullptr;
+    // Host copy, written by the finalize kernels: the head, and with host_data
+    // also max, argmax and sigma [S][K], the histograms [S][nbins] and the mean
+    // [K].  host_ready: the work that wrote it has completed.
+    bfi::HostHead* host = nullptr;
+    bool host_data = false, host_ready = false;
+    float* host_vmax() const { return reinterpret_cast<float*>(reinterpret_cast<char*>(host) + 64); }
+    int32_t* host_argmax() const { return reinterpret_cast<int32_t*>(host_vmax() + n_series * K); }
+    float* host_sigma() const { return reinterpret_cast<float*>(host_argmax() + n_series * K); }
+    float* host_mean() const { return host_sigma() + n_series * K; }
+    uint32_t* host_hist() const { return reinterpret_cast<uint32_t*>(host_mean() + K); }
     unsigned int cand_cap = 0;
     uint64_t n_candidates = 0;
     float thr = 0;

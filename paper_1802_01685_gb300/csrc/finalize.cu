@@ -51,9 +51,15 @@ __global__ void k_finalize(const __grid_constant__ FinalizeParams p, uint32_t K,
         const unsigned long long key = f.packed[k];
         const float a = __uint_as_float((uint32_t)(key >> 32));
         const uint32_t tau = ~(uint32_t)(key & 0xFFFFFFFFull);
+        const float sg = (float)sqrt(f.sumsq[k] / (double)f.L);
         f.vmax[k] = a;
         f.argmax[k] = (int32_t)tau;
-        f.sigma[k] = (float)sqrt(f.sumsq[k] / (double)f.L);
+        f.sigma[k] = sg;
+        if (f.h_vmax) {
+            f.h_vmax[k] = a;
+            f.h_argmax[k] = (int32_t)tau;
+            f.h_sigma[k] = sg;
+        }
         if (f.hist) {
             int b = (int)floorf(a * (float)nbins);
             b = b < 0 ? 0 : (b > (int)nbins - 1 ? (int)nbins - 1 : b);
@@ -62,15 +68,23 @@ __global__ void k_finalize(const __grid_constant__ FinalizeParams p, uint32_t K,
     }
 }
 
-// vmax is [n_series][K]; the mean runs over series in a fixed order
-__global__ void k_mean_max(const float* __restrict__ vmax, uint32_t n_series, uint32_t K,
-                           float* __restrict__ mean)
+// The mean over series in a fixed order, and the host copy's share of the last
+// kernel: status words, mean, histograms (complete now).  A host that waits for
+// the stream then has the results without a copy: eight copies of a few KB, 12
+// us each, were half of a small call.
+__global__ void k_publish(const __grid_constant__ PublishParams p)
 {
-    for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < K; k += gridDim.x * blockDim.x) {
+    const uint64_t i0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x, step = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t k = i0; k < p.K; k += step) {
         double acc = 0.0;
-        for (uint32_t s = 0; s < n_series; ++s) acc += (double)vmax[(size_t)s * K + k];
-        mean[k] = (float)(acc / (double)n_series);
+        for (uint32_t s = 0; s < p.n_series; ++s) acc += (double)p.vmax[(size_t)s * p.K + k];
+        const float m = (float)(acc / (double)p.n_series);
+        p.mean[k] = m;
+        if (p.h_mean) p.h_mean[k] = m;
     }
+    if (p.hist)
+        for (uint64_t i = i0; i < p.n_hist; i += step) p.h_hist[i] = p.hist[i];
+    if (p.head && i0 == 0) *p.head = HostHead{*p.err, p.counts[0], p.counts[1]};
 }
 
 cudaError_t launch_finalize(const FinalizeParams& p, uint32_t K, uint32_t nbins, cudaStream_t s)
@@ -84,13 +98,12 @@ cudaError_t launch_finalize(const FinalizeParams& p, uint32_t K, uint32_t nbins,
     return cudaGetLastError();
 }
 
-cudaError_t launch_mean_max(const float* vmax, uint32_t n_series, uint32_t K, float* mean,
-                            cudaStream_t s)
+cudaError_t launch_publish(const PublishParams& p, cudaStream_t s)
 {
-    unsigned b = (K + 255) / 256;
+    const unsigned b = (p.K + 255) / 256;
     if (b == 0) return cudaSuccess;
     count_launches(1);
-    k_mean_max<<<b, 256, 0, s>>>(vmax, n_series, K, mean);
+    k_publish<<<b, 256, 0, s>>>(p);
     return cudaGetLastError();
 }
 

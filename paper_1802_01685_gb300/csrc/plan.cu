@@ -75,7 +75,7 @@ bf_status bf_plan_create(bf_ctx* ctx, const bf_bank* bank, const size_t* lengths
     p->lengths.assign(lengths, lengths + n_series);
     p->fs = fs;
     cudaStream_t strm = ctx->stream;
-    st = alloc_result(ctx, bank, o, p->lengths, fs, strm, &p->r);
+    st = alloc_result(ctx, bank, o, p->lengths, fs, strm, true, &p->r);
     if (st) return st;
     p->r->plan_owned = true;
     p->prep.resize(n_series);
@@ -188,33 +188,21 @@ bf_status bf_plan_run(bf_plan* p, const float* const* series, void* stream, cons
     for (size_t s = 0; s < p->lengths.size() && e == cudaSuccess; ++s)
         e = cudaMemcpyAsync(p->prep[s].x, series[s], p->lengths[s] * sizeof(float), cudaMemcpyDefault,
                             strm);
-    cudaEvent_t e0 = nullptr, e1 = nullptr;
-    if (sync) {
-        cudaEventCreate(&e0);
-        cudaEventCreate(&e1);
-        cudaEventRecord(e0, strm);
-    }
+    p->r->host_ready = false;               // this run rewrites it
+    p->r->n_candidates = 0;
+    if (sync) cudaEventRecord(ctx->ev[0], strm);
     if (e == cudaSuccess) e = cudaGraphLaunch(p->exec, strm);
     if (e == cudaSuccess) count_launches(p->launches_per_run);
-    if (sync) cudaEventRecord(e1, strm);
+    if (sync) cudaEventRecord(ctx->ev[1], strm);
     if (e == cudaSuccess && sync) e = cudaStreamSynchronize(strm);
     if (sync) {
         float ms = 0.f;
-        if (e == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
+        if (e == cudaSuccess) cudaEventElapsedTime(&ms, ctx->ev[0], ctx->ev[1]);
         p->r->kernel_ms = ms;
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
     }
     if (e != cudaSuccess) return cuda_fail(e, "plan run");
-    p->r->n_candidates = 0;
     if (sync) {
-        bf_status st = check_device_status(ctx);
-        if (st) return st;
-        unsigned int c = 0;
-        cudaMemcpy(&c, p->r->cand_count, sizeof c, cudaMemcpyDeviceToHost);
-        p->r->n_candidates = c;
-        st = check_canaries(p->r);              // debug builds
-        if (st == BF_OK) st = result_status(p->r);      // non-finite samples
+        bf_status st = result_complete(p->r);
         if (st) return st;
     }
     *out = p->r;

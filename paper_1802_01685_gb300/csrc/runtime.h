@@ -76,7 +76,7 @@ int choose_lag_tile(bf_ctx* ctx, const Seg& g, int precision, cudaStream_t st);
 bf_status resolve_opts(const bf_bank* bank, const bf_opts* in, bf_opts* o);
 bf_status alloc_result(bf_ctx* ctx, const bf_bank* bank, const bf_opts& o,
                        const std::vector<size_t>& lengths, double fs, cudaStream_t st,
-                       bf_result** out);
+                       bool host_copy, bf_result** out);
 size_t result_bytes(const bf_bank* bank, const bf_opts& o, size_t N, double fs, size_t max_cand);
 bf_status finalize_result(bf_ctx* ctx, const bf_bank* bank, bf_result* r, cudaStream_t st);
 bf_status check_device_status(bf_ctx* ctx);
@@ -87,6 +87,10 @@ bf_status result_status(const bf_result* r);
 constexpr size_t CANARY_BYTES = 256;
 constexpr int CANARY_FILL = 0xA5;
 bf_status check_canaries(const bf_result* r);
+
+// the status of a search whose work has completed (BF_EDEVICE, BF_EINVAL for a
+// non-finite sample, canaries); on BF_OK its host copy is good to read
+bf_status result_complete(bf_result* r);
 
 void serve_shutdown(bf_ctx* ctx);
 

@@ -155,7 +155,7 @@ static bool admit(ServeState* S, Request* r)
     const bf_bank* bank = r->bank;
     std::vector<size_t> len{r->host.size()};
     bf_result* res = nullptr;
-    bf_status st = alloc_result(ctx, bank, r->opts, len, r->fs, S->stream, &res);
+    bf_status st = alloc_result(ctx, bank, r->opts, len, r->fs, S->stream, true, &res);
     if (st == BF_OK) {
         st = prepare_series(ctx, r->host.data(), r->host.size(), bank->M, bank->M_pad,
                             r->opts.precision, S->stream, &r->prep, res->status);
@@ -515,10 +515,9 @@ static void scheduler(ServeState* S)
                 continue;
             }
             if (!done_now.empty()) {
-                // a kernel that gave up on a wait marks every request it served
-                const bf_status dev = check_device_status(ctx);
                 std::lock_guard<std::mutex> g(S->mu);
                 const double t = now_s();
+                bf_status dev = BF_OK;
                 for (Request* r : done_now) {
                     S->active.erase(std::find(S->active.begin(), S->active.end(), r));
                     release_request_device(ctx, r);
@@ -529,21 +528,20 @@ static void scheduler(ServeState* S)
                         ++S->cancelled;
                         continue;
                     }
-                    // the candidate count, then the status word (non-finite samples)
-                    unsigned int w[2] = {0, 0};
-                    if (r->status == BF_OK && dev == BF_OK &&
-                        cudaMemcpy(w, r->result->cand_count, sizeof w, cudaMemcpyDeviceToHost) != cudaSuccess)
-                        r->status = BF_ECUDA;
-                    if (r->status == BF_OK && dev == BF_OK && (w[1] & 1u)) {
-                        r->status = BF_EINVAL;
-                        r->error = "the request's series holds a non-finite sample (NaN or infinity)";
+                    // a kernel that gave up on a wait marks every request it served
+                    // from then on, through the context's word; then the request's
+                    // own words (non-finite samples, candidates)
+                    if (r->status == BF_OK) {
+                        r->status = dev != BF_OK ? dev : result_complete(r->result);
+                        if (r->status == BF_EDEVICE) dev = BF_EDEVICE;
+                        if (r->status == BF_EINVAL)
+                            r->error = "the request's series holds a non-finite sample (NaN or infinity)";
                     }
-                    if (r->status != BF_OK || dev != BF_OK) {
+                    if (r->status != BF_OK) {
                         bf_result_destroy(r->result);
                         r->result = nullptr;
                         r->state = R_FAILED;
                     } else {
-                        r->result->n_candidates = w[0];
                         r->state = R_DONE;
                         r->t_done = t;
                         ++S->completed;
