@@ -451,12 +451,32 @@ int choose_lag_tile(bf_ctx* ctx, const Seg& g, int precision, cudaStream_t st)
     return best;
 }
 
+// Whether 256-lag tiles run in halves, each on a CTA of its own.  A launch takes
+// as many rounds as the busiest SM has tiles; a half costs HALF_COST of half a
+// tile: 60.3 ms against 48.4 on 64 s x 16,384 templates, its N = 128 MMAs read
+// the template operand for half the lags, which takes all of shared memory's
+// bandwidth.  So halves pay where whole tiles leave many SMs idle, on up to 76
+// tiles (a 4 s search of 256 templates, 50 tiles, went from 110 to 100 us) or
+// just past a full round.  Every output has the same MMA sequence either way.
+constexpr double HALF_COST = 1.25;
+
+static bool half_tiles(const std::vector<Seg>& segs, int n_sm)
+{
+    uint64_t whole = 0, half = 0;
+    for (const Seg& g : segs) {
+        whole += ceil_div(g.L, TC_TILE_L / 2) * g.n_tt;
+        half += ceil_div(g.L, TC_TILE_L / 4) * g.n_tt;
+    }
+    return HALF_COST * (double)ceil_div(half, n_sm) < 2.0 * (double)ceil_div(whole, n_sm);
+}
+
 cudaError_t launch_segments(bf_ctx* ctx, const std::vector<Seg>& segs, int precision, float thr,
                             Candidate* cand, unsigned int* cand_count, unsigned int cand_cap,
                             cudaStream_t st, uint64_t* tiles_out, int lt)
 {
     if (precision != BF_FP32 && lt == 0 && !segs.empty()) lt = choose_lag_tile(ctx, segs[0], precision, st);
     if (precision == BF_FP32) lt = SIMT_TILE_L;
+    else if (lt == TC_TILE_L / 2 && half_tiles(segs, ctx->n_sm)) lt = TC_TILE_L / 4;
     uint64_t tiles = 0;
     for (size_t b = 0; b < segs.size(); b += MAX_SEG) {
         CorrParams p{};

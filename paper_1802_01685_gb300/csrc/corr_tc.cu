@@ -45,11 +45,14 @@ constexpr uint32_t round1k(uint32_t b) { return (b + 1023u) & ~1023u; }
 // accumulator of 512 columns (two N = 256 MMAs per step) fills TMEM, and the
 // next tile's MMAs wait for the epilogue.  LT = 256: two accumulators of 256
 // columns used alternately, so the epilogue of one tile overlaps the MMAs of
-// the next, at twice the template-operand traffic per lag.
+// the next, at twice the template-operand traffic per lag.  LT = 128: half a
+// 256-lag tile (N = 128 MMAs), so that two CTAs share a tile where there are
+// few (half_tiles below).
 template <int LT>
 struct Geo {
-    static constexpr uint32_t NSUB = LT / 256;                 // N = 256 MMAs per step
-    static constexpr uint32_t NBUF = 512 / LT;                 // accumulators in TMEM
+    static constexpr uint32_t MMA_N = LT < 256 ? LT : 256;
+    static constexpr uint32_t NSUB = LT / MMA_N;               // MMAs per step
+    static constexpr uint32_t NBUF = LT == 512 ? 1 : 2;        // accumulators in TMEM, 256 columns apart
     static constexpr uint32_t B_ROWS = LT + TC_BK - 8;         // split rows per stage
     static constexpr uint32_t B_BYTES = B_ROWS * 16;
     static constexpr uint32_t OFF_AHI = 0;
@@ -69,7 +72,8 @@ constexpr uint64_t TIMEOUT_NS = 10ull * 1000 * 1000 * 1000;
 constexpr uint32_t TMEM_COLS = 512;
 
 // instruction descriptors, kind::f16, D = F32, both operands K-major, N = 256,
-// M = 128: A = B = BF16 (formats 1), or A = B = FP16 (formats 0)
+// M = 128: A = B = BF16 (formats 1), or A = B = FP16 (formats 0); the half tiles
+// put their N in its place
 constexpr uint32_t IDESC_BF16 = (1u << 4) | (1u << 7) | (1u << 10) | ((256u >> 3) << 17) |
                                 ((128u >> 4) << 24);
 constexpr uint32_t IDESC_F16 = (1u << 4) | ((256u >> 3) << 17) | ((128u >> 4) << 24);
@@ -443,6 +447,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_corr_tc(const __grid_constant
     const uint32_t drain_bar = bar0 + 8 * (2 * G::STAGES + 2 * G::NBUF);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t idesc = (p.idesc & ~(0x3fu << 17)) | ((G::MMA_N >> 3) << 17);
 
     if (threadIdx.x == 0) {
         for (uint32_t st = 0; st < G::STAGES; ++st) {
@@ -555,10 +560,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_corr_tc(const __grid_constant
                                 const uint64_t bhi = make_desc(sbase + G::OFF_BHI + boff, 128, 128);
                                 const uint64_t blo = make_desc(sbase + G::OFF_BLO + boff, 128, 128);
                                 const uint32_t d = tmem + b * 256 + h * 256;
-                                mma_f16(d, ahi, bhi, p.idesc, (kb != kb0) | (kk != 0));
+                                mma_f16(d, ahi, bhi, idesc, (kb != kb0) | (kk != 0));
                                 if (NPROD == 3) {
-                                    mma_f16(d, ahi, blo, p.idesc, 1);
-                                    mma_f16(d, alo, bhi, p.idesc, 1);
+                                    mma_f16(d, ahi, blo, idesc, 1);
+                                    mma_f16(d, alo, bhi, idesc, 1);
                                 }
                             }
                         }
@@ -748,6 +753,8 @@ cudaError_t corr_tc_set_attributes()
     cudaError_t e = set_attr<1, 512>();
     if (e == cudaSuccess) e = set_attr<1, 256>();
     if (e == cudaSuccess) e = set_attr<3, 256>();
+    if (e == cudaSuccess) e = set_attr<1, 128>();
+    if (e == cudaSuccess) e = set_attr<3, 128>();
     if (e == cudaSuccess) g_attr_done = true;
     return e;
 }
@@ -794,9 +801,12 @@ cudaError_t launch_corr_tc(const CorrParams& p, int nprod, int lt, int n_sm, cud
     const unsigned grid = (unsigned)(p.total_tiles < (uint64_t)n_sm ? p.total_tiles : (uint64_t)n_sm);
     count_launches(1);
     // the split routes need the second accumulator for their K chunks, so
-    // they run the 256-lag shape only
-    if (nprod == 3 && lt != 256) return cudaErrorInvalidValue;
-    if (lt == 256) {
+    // they run the 256-lag shape, whole or in halves, only
+    if (nprod == 3 && lt != 256 && lt != 128) return cudaErrorInvalidValue;
+    if (lt == 128) {
+        if (nprod == 3) k_corr_tc<3, 128><<<grid, TC_THREADS, Geo<128>::SMEM, st>>>(p);
+        else k_corr_tc<1, 128><<<grid, TC_THREADS, Geo<128>::SMEM, st>>>(p);
+    } else if (lt == 256) {
         if (nprod == 3) k_corr_tc<3, 256><<<grid, TC_THREADS, Geo<256>::SMEM, st>>>(p);
         else k_corr_tc<1, 256><<<grid, TC_THREADS, Geo<256>::SMEM, st>>>(p);
     } else {
