@@ -451,23 +451,20 @@ int choose_lag_tile(bf_ctx* ctx, const Seg& g, int precision, cudaStream_t st)
     return best;
 }
 
-// Whether 256-lag tiles run in halves, each on a CTA of its own.  A launch takes
-// as many rounds as the busiest SM has tiles; a half costs HALF_COST of half a
-// tile: 60.3 ms against 48.4 on 64 s x 16,384 templates, its N = 128 MMAs read
-// the template operand for half the lags, which takes all of shared memory's
-// bandwidth.  So halves pay where whole tiles leave many SMs idle, on up to 76
-// tiles (a 4 s search of 256 templates, 50 tiles, went from 110 to 100 us) or
-// just past a full round.  Every output has the same MMA sequence either way.
-constexpr double HALF_COST = 1.25;
-
-static bool half_tiles(const std::vector<Seg>& segs, int n_sm)
+// How many of a launch's 256-lag tiles run whole; the others run in halves, each
+// half on a CTA of its own, in a launch after it.  The persistent CTAs take tiles
+// in rounds of n_sm; a last round of at most half as many tiles leaves half the
+// SMs idle for a tile's time, and takes 0.62 of it in halves (N = 128 MMAs read
+// the template operand for half the lags, at shared memory's full bandwidth:
+// 60.3 ms against 48.4 for 64 s x 16,384 templates all in halves).  Where there
+// are whole tiles too, the second launch must be worth its few microseconds:
+// templates of 1024 samples or more, whose tiles take 12 us or more.  Every output
+// has the same MMA sequence either way.  A 4 s search of 256 templates (50 tiles)
+// went from 105 to 96 us, a mix of six served requests from 3.28 to 3.25 ms.
+static uint64_t whole_tiles(uint64_t tiles, uint32_t M_pad, int n_sm)
 {
-    uint64_t whole = 0, half = 0;
-    for (const Seg& g : segs) {
-        whole += ceil_div(g.L, TC_TILE_L / 2) * g.n_tt;
-        half += ceil_div(g.L, TC_TILE_L / 4) * g.n_tt;
-    }
-    return HALF_COST * (double)ceil_div(half, n_sm) < 2.0 * (double)ceil_div(whole, n_sm);
+    const uint64_t rest = tiles % (uint64_t)n_sm;
+    return 2 * rest <= (uint64_t)n_sm && (tiles == rest || M_pad >= 1024) ? tiles - rest : tiles;
 }
 
 cudaError_t launch_segments(bf_ctx* ctx, const std::vector<Seg>& segs, int precision, float thr,
@@ -476,7 +473,6 @@ cudaError_t launch_segments(bf_ctx* ctx, const std::vector<Seg>& segs, int preci
 {
     if (precision != BF_FP32 && lt == 0 && !segs.empty()) lt = choose_lag_tile(ctx, segs[0], precision, st);
     if (precision == BF_FP32) lt = SIMT_TILE_L;
-    else if (lt == TC_TILE_L / 2 && half_tiles(segs, ctx->n_sm)) lt = TC_TILE_L / 4;
     uint64_t tiles = 0;
     for (size_t b = 0; b < segs.size(); b += MAX_SEG) {
         CorrParams p{};
@@ -497,9 +493,16 @@ cudaError_t launch_segments(bf_ctx* ctx, const std::vector<Seg>& segs, int preci
         p.idesc = tc_idesc(precision);
         // accumulator chunks of 2048 samples (split-BF16) or 1024 (split-FP16)
         p.kchunk_log2 = precision == BF_SPLIT_FP16 ? 4u : 5u;
-        cudaError_t e = precision == BF_FP32 ? launch_corr_simt(p, st)
-                                             : launch_corr_tc(p, precision == BF_BF16 ? 1 : 3,
-                                                              lt, ctx->n_sm, st);
+        if (precision != BF_FP32 && lt == TC_TILE_L / 2) {
+            p.first = whole_tiles(t, p.seg[0].M_pad, ctx->n_sm);
+            p.total_tiles = p.first;
+        }
+        const int nprod = precision == BF_BF16 ? 1 : 3;
+        cudaError_t e = precision == BF_FP32 ? launch_corr_simt(p, st) : launch_corr_tc(p, nprod, lt, ctx->n_sm, st);
+        if (e == cudaSuccess && p.first < t && precision != BF_FP32 && lt == TC_TILE_L / 2) {
+            p.total_tiles = 2 * (t - p.first);
+            e = launch_corr_tc(p, nprod, TC_TILE_L / 4, ctx->n_sm, st);
+        }
         if (e != cudaSuccess) return e;
         tiles += t;
     }

@@ -112,7 +112,8 @@ struct Seg {
 struct CorrParams {
     int n_seg;
     uint32_t idesc;                 // tcgen05 instruction descriptor (operand type)
-    uint64_t total_tiles;
+    uint64_t total_tiles;           // items of the launch
+    uint64_t first;                 // launches of half tiles: the first tile that runs in halves
     float thr;                      // candidate threshold on |rho|
     unsigned int cand_cap;
     Candidate* cand;

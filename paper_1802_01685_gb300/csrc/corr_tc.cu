@@ -47,7 +47,7 @@ constexpr uint32_t round1k(uint32_t b) { return (b + 1023u) & ~1023u; }
 // columns used alternately, so the epilogue of one tile overlaps the MMAs of
 // the next, at twice the template-operand traffic per lag.  LT = 128: half a
 // 256-lag tile (N = 128 MMAs), so that two CTAs share a tile where there are
-// few (half_tiles below).
+// few (p.first, whole_tiles in api.cu).
 template <int LT>
 struct Geo {
     static constexpr uint32_t MMA_N = LT < 256 ? LT : 256;
@@ -413,15 +413,19 @@ __device__ __forceinline__ KRange chunk_range(KRange kr, uint32_t ch, uint32_t l
     return {max(kr.lo, a), min(kr.hi, a + (1u << lg))};
 }
 
+// Item t of the launch: tile t, or with LT = 128 one half of the 256-lag tile
+// p.first + t / 2 (the second half may hold no lag).
 template <int LT>
 __device__ __forceinline__ TileCoord tile_coord(const CorrParams& p, uint64_t t)
 {
-    const Seg* s = &p.seg[find_seg(p, t)];
-    const uint64_t local = t - s->tile_begin;
+    constexpr bool HALF = LT == 128;
+    const uint64_t tile = HALF ? p.first + (t >> 1) : t;
+    const Seg* s = &p.seg[find_seg(p, tile)];
+    const uint64_t local = tile - s->tile_begin;
     TileCoord c;
     c.s = s;
     c.tt = s->tt0 + (uint32_t)(local / s->n_lag_tiles);
-    c.lag0 = (uint32_t)(local % s->n_lag_tiles) * LT;
+    c.lag0 = (uint32_t)(local % s->n_lag_tiles) * (HALF ? 256 : LT) + (HALF ? (uint32_t)(t & 1) * LT : 0u);
     return c;
 }
 
@@ -447,7 +451,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_corr_tc(const __grid_constant
     const uint32_t drain_bar = bar0 + 8 * (2 * G::STAGES + 2 * G::NBUF);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t idesc = (p.idesc & ~(0x3fu << 17)) | ((G::MMA_N >> 3) << 17);
+    const uint32_t idesc = LT < 256 ? (p.idesc & ~(0x3fu << 17)) | ((G::MMA_N >> 3) << 17) : p.idesc;
 
     if (threadIdx.x == 0) {
         for (uint32_t st = 0; st < G::STAGES; ++st) {
@@ -590,7 +594,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_corr_tc(const __grid_constant
         for (uint64_t t = blockIdx.x; t < p.total_tiles; t += gridDim.x) {
             const TileCoord c = tile_coord<LT>(p, t);
             const Seg& s = *c.s;
-            const uint32_t nvalid = min((uint32_t)LT, s.L - c.lag0);
+            const uint32_t nvalid = LT == 128 && c.lag0 >= s.L ? 0u : min((uint32_t)LT, s.L - c.lag0);
             // split-FP16 operands were scaled by 2^s (series) and 2^8 (templates)
             const float oscale = s.xmax ? ldexpf(1.f, -(f16_series_shift(*s.xmax) + 8)) : 1.f;
             epilogue_sync();
