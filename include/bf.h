@@ -274,10 +274,10 @@ typedef struct {
                                 bf_result_get_sigma_pred)                      */
     int32_t tile_lags;       /* lags per tensor-core tile: 512 (one TMEM
                                 accumulator) or 256 (two, so the epilogue of
-                                   one tile overlaps the MMAs of the next; the
-                                   last tiles of a launch may run in two halves
-                                   on two SMs, with the same outputs); 0 =
-                                   chosen by the library's autotuner, which times
+                                one tile overlaps the MMAs of the next; the
+                                last tiles of a launch may run in two halves
+                                on two SMs, with the same outputs); 0 =
+                                chosen by the library's autotuner, which times
                                 both once per precision and template length
                                 per context.  Ignored by BF_FP32.            */
 } bf_opts;
