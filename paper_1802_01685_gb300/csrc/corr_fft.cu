@@ -760,6 +760,16 @@ __device__ __forceinline__ void rotate2(cpk& v, float2 wr, float2 wi)
     v.r = r;
 }
 
+// v *= w, one twiddle for both lanes: unpacked, as a packed FMA of three distinct
+// register pairs takes the time of two and the pairs (w, w) would have to be made
+__device__ __forceinline__ void rotate1(cpk& v, float2 w)
+{
+    const float ax = v.r.x * w.x - v.i.x * w.y, ay = v.r.y * w.x - v.i.y * w.y;
+    const float bx = v.r.x * w.y + v.i.x * w.x, by = v.r.y * w.y + v.i.y * w.x;
+    v.r = make_float2(ax, ay);
+    v.i = make_float2(bx, by);
+}
+
 // dft4<+1> and dft16<+1> on packed values
 __device__ __forceinline__ void dft4_pk(cpk& a, cpk& b, cpk& c, cpk& d)
 {
@@ -1071,7 +1081,7 @@ __global__ void __launch_bounds__(FT, 1) k_corr_fft(const __grid_constant__ FftP
                 for (int k1 = 0; k1 < 4; ++k1) {
                     if (k1 + k2 == 0) continue;
                     const float2 f = k1 == 0 ? u[k2] : k2 == 0 ? w[k1] : cmul(u[k2], w[k1]);
-                    rotate2(v[4 * k1 + k2], make_float2(f.x, f.x), make_float2(f.y, f.y));
+                    rotate1(v[4 * k1 + k2], f);
                 }
             bar_sync(BAR_G, GT);                          // 1: every warp is done with the work array
             float4* const zz = z + (j >> 4) * ZROW + (j & 15);
@@ -1090,7 +1100,7 @@ __global__ void __launch_bounds__(FT, 1) k_corr_fft(const __grid_constant__ FftP
                 const int q = (c >> 2) + 4 * (c & 3);
                 if (q) {
                     const float2 f = twb[(q - 1) * 16 + (tg & 15)];
-                    rotate2(v[c], make_float2(f.x, f.x), make_float2(f.y, f.y));
+                    rotate1(v[c], f);
                 }
                 zz[ZROW * q] = pack4(v[c]);
             }
