@@ -4,16 +4,20 @@
 //
 // Block tile: 64 templates x 256 lags, 256 threads.  Warp w owns templates
 // 8w .. 8w+7 of the tile; lane l owns the eight consecutive lags 8l .. 8l+7, so
-// one 32-sample chunk of the series (40 values per thread, held in registers)
-// slides under the eight template rows: 64 FMAs per template value pair and no
-// re-read of the series.  Templates come from the row-major FP32 layout.
+// twelve values of the series, held in registers, slide under four samples of
+// the eight template rows: 256 FMAs to nine 16-byte shared loads.  Templates
+// come from the row-major FP32 layout.
 //
 // Bound: FP32 FMA.  The next chunk arrives by cp.async in a second buffer while
-// this one is used, so a chunk costs one barrier and no wait for L2: 2 x 30,000
-// samples against 2048 templates of 2048 samples take 7.66 ms where staging
-// through registers between two barriers took 8.19 (59 -> 63 TFLOP/s of 78.5).
-// Packed FMAs (two lags a register pair) were slower, 8.3-9.1 ms: with three
-// distinct 64-bit operands they take three cycles, not two.
+// this one is used, so a chunk costs one barrier and no wait for L2, and four
+// samples of one template row are multiplied sample by sample over all lags:
+// 2 x 30,000 samples against 2048 templates of 2048 samples take 7.45 ms where
+// staging through registers between two barriers took 8.19 and a window of 40
+// values, lag by lag, 7.55 (59, 65 and 64 TFLOP/s of 78.5).  Slower: packed
+// FMAs (two lags a register pair), 8.3-9.1 ms, as with three distinct 64-bit
+// operands they take three cycles, not two; chunks of 64 samples, 9.8 (the
+// unrolled loop outgrows the instruction cache) or 8.2 rolled; 16 lags a
+// thread, 8.3-8.8.
 #include "corr_common.cuh"
 
 namespace bfi {
@@ -76,28 +80,34 @@ __global__ void __launch_bounds__(SIMT_THREADS, 2) k_corr_simt(const __grid_cons
             const float (&sh_t)[SIMT_TILE_T][SIMT_BK] = sh_t2[buf];
             const float (&sh_x)[XW] = sh_x2[buf];
 
-            float xr[40];
+            // the eight lags' values of the series slide four samples at a time
+            float xr[12];
 #pragma unroll
-            for (int q = 0; q < 10; ++q) {
-                float4 v = *reinterpret_cast<const float4*>(&sh_x[8 * lane + 4 * q]);
-                xr[4 * q + 0] = v.x;
-                xr[4 * q + 1] = v.y;
-                xr[4 * q + 2] = v.z;
-                xr[4 * q + 3] = v.w;
+            for (int q = 0; q < 8; q += 4) {
+                const float4 v = *reinterpret_cast<const float4*>(&sh_x[8 * lane + q]);
+                xr[q + 0] = v.x;
+                xr[q + 1] = v.y;
+                xr[q + 2] = v.z;
+                xr[q + 3] = v.w;
             }
 #pragma unroll
             for (int mm = 0; mm < SIMT_BK; mm += 4) {
+                const float4 v = *reinterpret_cast<const float4*>(&sh_x[8 * lane + mm + 8]);
+                xr[8] = v.x;
+                xr[9] = v.y;
+                xr[10] = v.z;
+                xr[11] = v.w;
 #pragma unroll
                 for (int a = 0; a < 8; ++a) {
-                    float4 hv = *reinterpret_cast<const float4*>(&sh_t[8 * warp + a][mm]);
+                    const float4 hv = *reinterpret_cast<const float4*>(&sh_t[8 * warp + a][mm]);
+                    const float h[4] = {hv.x, hv.y, hv.z, hv.w};
 #pragma unroll
-                    for (int b = 0; b < 8; ++b) {
-                        acc[a][b] = fmaf(hv.x, xr[b + mm + 0], acc[a][b]);
-                        acc[a][b] = fmaf(hv.y, xr[b + mm + 1], acc[a][b]);
-                        acc[a][b] = fmaf(hv.z, xr[b + mm + 2], acc[a][b]);
-                        acc[a][b] = fmaf(hv.w, xr[b + mm + 3], acc[a][b]);
-                    }
+                    for (int q = 0; q < 4; ++q)
+#pragma unroll
+                        for (int b = 0; b < 8; ++b) acc[a][b] = fmaf(h[q], xr[b + q], acc[a][b]);
                 }
+#pragma unroll
+                for (int u = 0; u < 8; ++u) xr[u] = xr[u + 4];
             }
         }
 
