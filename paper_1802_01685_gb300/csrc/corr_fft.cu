@@ -864,14 +864,17 @@ __device__ __forceinline__ float2 root64(int a)
 // row's before the other has passed this one's).  All waits are hardware
 // barriers between these two groups.
 //
-// What bounds it: the L1/shared-memory pipe, 4.7 K wavefronts a transform (the
-// spectra and norms 1.5 K, the work array 2 K, mirrors 0.3 K), beside 3.8 K
-// cycles of FP32 and 3.2 K of issue; a transform takes 7.3 K cycles.  On 16 s x
-// 4096 templates of 4096 samples (20,480 transforms) it runs 487 us; the form
-// it replaced (one CTA-wide group with the template in registers, unpacked
-// arithmetic, the radix-2 stage last through shared memory, 12.8 K warp
-// instructions more per transform and four CTA-wide barriers) ran 664 us.  The
-// 64 s x 4 series x 65,536 template step went from 163.7 to 121.6 ms.
+// What bounds it: the L1 data pipe, 4.7 K wavefronts a transform at five
+// segments a template (work array 2.2 K, spectra 1.5 K, norms, mirrors and
+// twiddles 1 K), beside 4.1 K cycles of FP32 and 3.9 K of issue (61, 53 and 50 %
+// busy).  A transform takes 7.7 K cycles (6.6 K at 84 segments a template): four
+// warps a scheduler do not overlap the three any further, and the registers and
+// the shared memory hold no third group.  16 s x 16,384 templates of 4096
+// samples (81,920 transforms) run 2.00 ms; the form it replaced (one CTA-wide
+// group with the template in registers, unpacked arithmetic, the radix-2 stage
+// last through shared memory, 9 K warp instructions more per transform and four
+// CTA-wide barriers) ran 2.60.  The 64 s x 4 series x 65,536 template step went
+// from 163.6 to 119.3 ms.  Unpacked twiddle products (rotate1) are 1 % of that.
 template <bool QUAD, bool DENSE>
 __global__ void __launch_bounds__(FT, 1) k_corr_fft(const __grid_constant__ FftParams p, uint32_t total)
 {
