@@ -143,6 +143,8 @@ bf_status bf_plan_create(bf_ctx* ctx, const bf_bank* bank, const size_t* lengths
     cudaError_t e = cudaStreamBeginCapture(strm, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamBeginCapture");
     cudaError_t ec = clear_result(p->r, strm);
+    // a generated bank's first chunk is made beside the preparation
+    if (ec == cudaSuccess && !fft && bank->generated) ec = gen_begin(ctx, bank, o, strm, ring);
     if (ec == cudaSuccess) {
         const std::vector<const PreparedSeries*> pp(pptr.begin(), pptr.end());
         ec = prepare_series_batch(pp, bank->M, o.precision, strm);
