@@ -46,7 +46,8 @@ constexpr uint32_t TILE_BYTES_A = TC_TILE_T * TC_BK * 2;   // 16 KiB per k-block
 
 // device error codes written to the context's status word
 enum : int { DEV_OK = 0, DEV_TIMEOUT_FULL = 1, DEV_TIMEOUT_EMPTY = 2,
-             DEV_TIMEOUT_TMEM = 3, DEV_TMEM_ALLOC = 4, DEV_BOUNDS = 5 };
+             DEV_TIMEOUT_TMEM = 3, DEV_TMEM_ALLOC = 4, DEV_BOUNDS = 5,
+             DEV_TIMEOUT_FFT = 6 };
 
 // Debug builds (-DBF_DEBUG_BOUNDS, built as libbf_debug.so): the kernels
 // check the indices their outputs, staging buffers and tables rely on --

@@ -82,7 +82,8 @@ static_assert(FFT_SMEM % 16 == 0 && (FFT_SMEM + ZPAD * sizeof(float2)) % 16 == 0
 constexpr int GT = FT / 2;
 constexpr int ZROW = 17, ZBLK = 16 * ZROW, ZG = 16 * ZBLK;
 constexpr int TWC_N = 6 * 256 + 15 * 16 + 2 * 256;          // float2 entries, after the TW_N of the forward transforms
-constexpr size_t CORR_SMEM = (size_t)(2 * ZG + FH + TWC_N / 2 + 2 * 9 + FT / 32) * sizeof(float4);   // 2 x 9: column 0; the warps' reductions
+// 2 x 9: column 0; the warps' reductions; two mbarriers
+constexpr size_t CORR_SMEM = (size_t)(2 * ZG + FH + TWC_N / 2 + 2 * 9 + FT / 32 + 1) * sizeof(float4);
 static_assert(CORR_SMEM <= 227 * 1024, "the correlation kernel fits one SM's shared memory");
 static_assert(TW_N % 2 == 0 && TWC_N % 2 == 0, "16-byte tables");
 
@@ -737,9 +738,13 @@ __device__ __forceinline__ void prefetch_l2(const void* g)
 // n = 256 n2 + 16 n1 + n0, pass 1 turns n2 into k0, pass 2 n1 into k1, pass 3
 // n0 into k2, k = k0 + 16 k1 + 256 k2, every thread writing back to the slots
 // it read, so one array serves.  Passes 2 and 3 of a block of equal k0 belong to
-// one half-warp: only pass 1 crosses warps, so a group meets at two barriers a
-// transform (before and after pass 1 writes) and its warps drift apart between
-// them, some in shared memory while others compute.
+// one half-warp: only pass 1 crosses warps, so a group meets at one barrier a
+// transform, after pass 1 writes.  That all its warps have read the transform
+// before is an mbarrier's: they arrive after pass 3's reads and wait before pass
+// 1's writes, long after, and so drift apart between the barriers, some in shared
+// memory while others compute.  With a barrier in the mbarrier's place a
+// transform took 3 % longer (16 s x 4096 templates in a plan: 541 us a run, 556
+// before).
 
 // two complex values, one per register half
 struct cpk {
@@ -827,6 +832,39 @@ __device__ __forceinline__ void bar_arrive(int id, int count)
     asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
 
+// A work array's mbarrier, of one phase a transform: the group's warps arrive
+// when they have read their last of the transform from it, and wait for all
+// before they write the next one's.  The wait is bounded (seconds, against the
+// microseconds that it takes); on expiry the status word is set and the kernel
+// goes on, so that it ends.
+__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count)
+{
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"((unsigned)__cvta_generic_to_shared(bar)), "r"(count)
+                 : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar)
+{
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0)
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"((unsigned)__cvta_generic_to_shared(bar))
+                     : "memory");
+}
+__device__ __forceinline__ void mbar_wait(uint64_t* bar, uint32_t parity, int* err)
+{
+    const unsigned a = (unsigned)__cvta_generic_to_shared(bar);
+    for (int n = 0; n < (1 << 22); ++n) {
+        uint32_t done;
+        asm volatile("{\n\t.reg .pred p;\n\t"
+                     "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                     "selp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(done)
+                     : "r"(a), "r"(parity)
+                     : "memory");
+        if (done) return;
+    }
+    if (err) atomicCAS(err, DEV_OK, DEV_TIMEOUT_FFT);
+}
+
 // e^{i pi a / 32} for a compile-time a in [0, 8)
 __device__ __forceinline__ float2 root64(int a)
 {
@@ -861,8 +899,8 @@ __device__ __forceinline__ float2 root64(int a)
 // the group with the row's last item fetches the next row's spectra during
 // its first two passes and then opens them to the other group (barrier FULL,
 // of two that alternate with the row: the fetching group may reach the next
-// row's before the other has passed this one's).  All waits are hardware
-// barriers between these two groups.
+// row's before the other has passed this one's).  All these
+// are hardware barriers.
 //
 // What bounds it: the L1 data pipe, 4.7 K wavefronts a transform at five
 // segments a template (work array 2.2 K, spectra 1.5 K, norms, mirrors and
@@ -874,7 +912,7 @@ __device__ __forceinline__ float2 root64(int a)
 // group with the template in registers, unpacked arithmetic, the radix-2 stage
 // last through shared memory, 9 K warp instructions more per transform and four
 // CTA-wide barriers) ran 2.60.  The 64 s x 4 series x 65,536 template step went
-// from 163.6 to 119.3 ms.  Unpacked twiddle products (rotate1) are 1 % of that.
+// from 163.6 to 115.4 ms.  Unpacked twiddle products (rotate1) are 1 % of that.
 template <bool QUAD, bool DENSE>
 __global__ void __launch_bounds__(FT, 1) k_corr_fft(const __grid_constant__ FftParams p, uint32_t total)
 {
@@ -897,6 +935,8 @@ __global__ void __launch_bounds__(FT, 1) k_corr_fft(const __grid_constant__ FftP
         double ss;
     };
     Acc& acc = reinterpret_cast<Acc*>(h + FH + TWC_N / 2 + 2 * 9)[threadIdx.x >> 5];
+    // the group's mbarrier: its work array is read
+    uint64_t* const zread = reinterpret_cast<uint64_t*>(h + FH + TWC_N / 2 + 2 * 9 + FT / 32) + g;
     const int BAR_G = 1 + g, BAR_EMPTY = 3, BAR_FULL = 4;          // FULL: two, by the parity of the row
     constexpr uint32_t BINS = QUAD ? FH : FN;             // complex bins per segment
     constexpr uint32_t KR = QUAD ? 2 : 1;                 // template rows per item
@@ -911,6 +951,7 @@ __global__ void __launch_bounds__(FT, 1) k_corr_fft(const __grid_constant__ FftP
     auto spectra = [&](uint32_t row) {
         return reinterpret_cast<const float4*>(p.hspec + (size_t)(p.k_lo + row * KR - p.hrow0) * BINS);
     };
+    if (tg == 0) mbar_init(zread, GT / 32);
     {
         const float4* src = reinterpret_cast<const float4*>(p.tw + TW_N);
         for (int e = threadIdx.x; e < TWC_N / 2; e += FT) cp_async16(h + FH + e, src + e);
@@ -1086,12 +1127,14 @@ __global__ void __launch_bounds__(FT, 1) k_corr_fft(const __grid_constant__ FftP
                     const float2 f = k1 == 0 ? u[k2] : k2 == 0 ? w[k1] : cmul(u[k2], w[k1]);
                     rotate1(v[4 * k1 + k2], f);
                 }
-            bar_sync(BAR_G, GT);                          // 1: every warp is done with the work array
+            // every warp has read the transform before (item / 2 of them) from the work array
+            mbar_wait(zread, ((item >> 1) & 1) ^ 1, p.err);
+            __syncwarp();
             float4* const zz = z + (j >> 4) * ZROW + (j & 15);
 #pragma unroll
             for (int c = 0; c < 16; ++c) zz[((c >> 2) + 4 * (c & 3)) * ZBLK] = pack4(v[c]);
         }
-        bar_sync(BAR_G, GT);                              // 2: pass 1 is written
+        bar_sync(BAR_G, GT);                              // pass 1 is written
         {
             // pass 2: thread (k0, n0) = (tg / 16, tg % 16); twiddle e^{2 pi i q n0 / 256}
             float4* const zz = z + (tg >> 4) * ZBLK + (tg & 15);
@@ -1119,6 +1162,7 @@ __global__ void __launch_bounds__(FT, 1) k_corr_fft(const __grid_constant__ FftP
 #pragma unroll
             for (int r = 0; r < 16; ++r) v[r] = unpack4(zz[r]);
         }
+        mbar_arrive(zread);
         // norms of the lags of this thread's output q: lags 4 k .. 4 k + 3 in the order
         // 0, 2, 1, 3 (real route), lags 2 k, 2 k + 1 (pair route), stored by (q, tg);
         // zero past the segment's end
