@@ -740,8 +740,8 @@ __device__ __forceinline__ void prefetch_l2(const void* g)
 // it read, so one array serves.  Passes 2 and 3 of a block of equal k0 belong to
 // one half-warp: only pass 1 crosses warps, so a group meets at one barrier a
 // transform, after pass 1 writes.  That all its warps have read the transform
-// before is an mbarrier's: they arrive after pass 3's reads and wait before pass
-// 1's writes, long after, and so drift apart between the barriers, some in shared
+// before is an mbarrier's: they arrive after pass 3's reads and wait before the
+// next pass 1, long after, and so drift apart between the barriers, some in shared
 // memory while others compute.  With a barrier in the mbarrier's place a
 // transform took 3 % longer (16 s x 4096 templates in a plan: 541 us a run, 556
 // before).
@@ -1110,6 +1110,10 @@ __global__ void __launch_bounds__(FT, 1) k_corr_fft(const __grid_constant__ FftP
                 departed = true;
             }
         }
+        // every warp has read the transform before (item / 2 of them) from the work
+        // array; asked for here, ahead of the arithmetic, and not at the writes (1 %)
+        mbar_wait(zread, ((item >> 1) & 1) ^ 1, p.err);
+        __syncwarp();
         // pass 1: out k0 = q at position 4 k1 + k2 of dft16, q = k1 + 4 k2; twiddle e^{2 pi i q j / 4096}
         dft16_pk(v);
         {
@@ -1127,9 +1131,6 @@ __global__ void __launch_bounds__(FT, 1) k_corr_fft(const __grid_constant__ FftP
                     const float2 f = k1 == 0 ? u[k2] : k2 == 0 ? w[k1] : cmul(u[k2], w[k1]);
                     rotate1(v[4 * k1 + k2], f);
                 }
-            // every warp has read the transform before (item / 2 of them) from the work array
-            mbar_wait(zread, ((item >> 1) & 1) ^ 1, p.err);
-            __syncwarp();
             float4* const zz = z + (j >> 4) * ZROW + (j & 15);
 #pragma unroll
             for (int c = 0; c < 16; ++c) zz[((c >> 2) + 4 * (c & 3)) * ZBLK] = pack4(v[c]);
@@ -1172,7 +1173,7 @@ __global__ void __launch_bounds__(FT, 1) k_corr_fft(const __grid_constant__ FftP
             const float2 f = __ldg(reinterpret_cast<const float2*>(nrm) + GT * q + tg);
             return make_float4(f.x, f.y, 0.f, 0.f);
         };
-        constexpr int AHEAD = 6;
+        constexpr int AHEAD = 7;
         float4 iv[AHEAD];
 #pragma unroll
         for (int q = 0; q < AHEAD; ++q) iv[q] = norms(q);
