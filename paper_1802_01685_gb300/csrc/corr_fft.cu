@@ -412,6 +412,17 @@ __device__ __forceinline__ void quad_bins(const float2* z, float2 base_f, int i,
     u[3] = make_float2(c.x - vr, c.y - vi);
 }
 
+// The place of column j among a row's 256 records: that of the thread which reads
+// it in the correlation kernel, whose lanes 16-31 hold the mirrors of lanes
+// 0-15's columns, so that a warp reads 512 bytes in a row.  In the order of j the
+// mirrors' 256 bytes lay across three lines, one of them shared with the warp
+// beside (3 % on the light curves, 0.5-1 % elsewhere).
+__device__ __forceinline__ int record_place(int j)
+{
+    const int m = j < GT / 2 ? j : GT - j;            // a mirror's column: 1 .. 127; 128 is in the place of 0's
+    return j == GT / 2 ? 16 : 32 * (m >> 4) + (j < GT / 2 ? 0 : 16) + (m & 15);
+}
+
 __device__ __forceinline__ float4 lanes(float2 a, float2 b) { return make_float4(a.x, b.x, a.y, b.y); }
 
 // S[k] and S[N - k] from U[k] and U[N - k], w = e^{i pi k / N} (real_spectrum)
@@ -425,15 +436,15 @@ __device__ __forceinline__ void real_split(float2 uk, float2 um, float2 w, float
 }
 
 // The half spectrum of a real signal (as real_spectrum) as the records the
-// correlation kernel reads: for n = j + 256 r < 2048, float4 number 2 r 256 + j
-// holds the bins n and 4096 - n as (re, re, im, im), number (2 r + 1) 256 + j the
-// bins 8192 - n and 4096 + n; the record of n = 0 holds bin 0 = (S[0], S[N]), bin
+// correlation kernel reads: for n = j + 256 r < 2048, float4 number 2 r 256 +
+// record_place(j) holds the bins n and 4096 - n as (re, re, im, im), number
+// (2 r + 1) 256 + record_place(j) the bins 8192 - n and 4096 + n; the record of n = 0 holds bin 0 = (S[0], S[N]), bin
 // 4096, bin 6144 and bin 2048.
 __device__ __forceinline__ void real_spectrum_quads(const Smem& m, float2 base_f, float2 base_r,
                                                     float2* __restrict__ out)
 {
     const int tid = threadIdx.x;
-    float4* rec = reinterpret_cast<float4*>(out) + 2 * GT * (tid / GT) + tid % GT;
+    float4* rec = reinterpret_cast<float4*>(out) + 2 * GT * (tid / GT) + record_place(tid % GT);
 #pragma unroll
     for (int i = 0; i < FBINS / 2; ++i) {
         float2 u[4], s0, s1, s2, s3;                  // bins n, 4096 - n, 8192 - n, 4096 + n
@@ -455,8 +466,8 @@ __device__ __forceinline__ void real_spectrum_quads(const Smem& m, float2 base_f
 
 // Spectra of segments of a batch of series, as the correlation kernel's
 // records.  Pair route (F = 8192): the real segment through one complex
-// transform, 4096 bins: for n = j + 256 r < 2048, float4 number r 256 + j holds
-// the bins n and 4096 - n (for n = 0: bin 0 = (DC, Nyquist) and bin 2048).  Real
+// transform, 4096 bins: for n = j + 256 r < 2048, float4 number r 256 +
+// record_place(j) holds the bins n and 4096 - n (for n = 0: bin 0 = (DC, Nyquist) and bin 2048).  Real
 // route (F = 16384): even/odd packed, 8192 bins (real_spectrum_quads).
 template <bool REAL>
 __global__ void __launch_bounds__(FT, 1) k_fft_series(const __grid_constant__ FftSeriesBatch p,
@@ -486,7 +497,7 @@ __global__ void __launch_bounds__(FT, 1) k_fft_series(const __grid_constant__ Ff
         if (REAL) {
             real_spectrum_quads(m, base_f, base_r, p.spec[s] + (size_t)j * FN);
         } else {
-            float4* rec = reinterpret_cast<float4*>(p.spec[s] + (size_t)j * FH) + tid;
+            float4* rec = reinterpret_cast<float4*>(p.spec[s] + (size_t)j * FH) + GT * (tid / GT) + record_place(tid % GT);
 #pragma unroll
             for (int i = 0; i < FBINS / 2; ++i) {
                 float2 u[4];
@@ -517,8 +528,8 @@ __global__ void __launch_bounds__(FT, 1) k_fft_bank_pair(const float* __restrict
         for (int n = tid; n < FN; n += FT) m.z[n + (n >> 4)] = make_float2(ra[n], b < n_rows ? rb[n] : 0.f);
         __syncthreads();
         fft_passes<-1>(m);
-        float4* sa = reinterpret_cast<float4*>(spec + (size_t)a * FH) + tid;
-        float4* sb = reinterpret_cast<float4*>(spec + (size_t)b * FH) + tid;
+        float4* sa = reinterpret_cast<float4*>(spec + (size_t)a * FH) + GT * (tid / GT) + record_place(tid % GT);
+        float4* sb = reinterpret_cast<float4*>(spec + (size_t)b * FH) + GT * (tid / GT) + record_place(tid % GT);
 #pragma unroll
         for (int i = 0; i < FBINS / 2; ++i) {
             float2 u[4];                           // Z[n], Z[n + 4096], Z[4096 - n], Z[8192 - n]
@@ -865,6 +876,16 @@ __device__ __forceinline__ void mbar_wait(uint64_t* bar, uint32_t parity, int* e
     if (err) atomicCAS(err, DEV_OK, DEV_TIMEOUT_FFT);
 }
 
+// 16 bytes of global memory past L1: the norms, which would displace the segment
+// spectra there (light curves 8.43 -> 8.27 ms, a 16 s plan 529 -> 526 us, the 64 s
+// step 7.32 -> 7.38 ms; the spectra themselves past L1 cost 4 % there)
+__device__ __forceinline__ float4 ldg_past_l1(const float4* p)
+{
+    float4 f;
+    asm("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(f.x), "=f"(f.y), "=f"(f.z), "=f"(f.w) : "l"(p));
+    return f;
+}
+
 // e^{i pi a / 32} for a compile-time a in [0, 8)
 __device__ __forceinline__ float2 root64(int a)
 {
@@ -887,13 +908,14 @@ __device__ __forceinline__ float2 root64(int a)
 // into registers.
 //
 // Spectra are kept as records (see real_spectrum_quads): float4 number
-// (2 r + side) 256 + j (real route) or r 256 + j (pair route) holds, for
-// n = j + 256 r, the bins n and 4096 - n (side 0), 8192 - n and 4096 + n
-// (side 1), as (re, re, im, im).  One record gives Z[n], Z[n + 4096], and their
-// mirrors Z[4096 - n], Z[8192 - n]: the packed inputs n and 4096 - n of the
-// transform.  The second belongs to the thread of 256 - j, which sits 16 lanes
-// away in the same warp: lanes 0-15 of warp w hold j = 16 w + lane, lanes 16-31
-// 256 - j of them (and 128 in the place of 0's, both being their own mirrors).
+// (2 r + side) 256 + t (real route) or r 256 + t (pair route) is thread t's; for
+// its column j (record_place(j) = t) and n = j + 256 r it holds the bins n and
+// 4096 - n (side 0), 8192 - n and 4096 + n (side 1), as (re, re, im, im).  One
+// record gives Z[n], Z[n + 4096], and their mirrors Z[4096 - n], Z[8192 - n]:
+// the packed inputs n and 4096 - n of the transform.  The second belongs to the
+// thread of 256 - j, which sits 16 lanes away in the same warp: lanes 0-15 of
+// warp w hold j = 16 w + lane, lanes 16-31 256 - j of them (and 128 in the place
+// of 0's, both being their own mirrors).
 //
 // When both groups have formed their last product of a row (barrier EMPTY),
 // the group with the row's last item fetches the next row's spectra during
@@ -908,11 +930,11 @@ __device__ __forceinline__ float2 root64(int a)
 // busy).  A transform takes 7.7 K cycles (6.6 K at 84 segments a template): four
 // warps a scheduler do not overlap the three any further, and the registers and
 // the shared memory hold no third group.  16 s x 16,384 templates of 4096
-// samples (81,920 transforms) run 2.00 ms; the form it replaced (one CTA-wide
+// samples (81,920 transforms) run 1.94 ms; the form it replaced (one CTA-wide
 // group with the template in registers, unpacked arithmetic, the radix-2 stage
 // last through shared memory, 9 K warp instructions more per transform and four
 // CTA-wide barriers) ran 2.60.  The 64 s x 4 series x 65,536 template step went
-// from 163.6 to 115.4 ms.  Unpacked twiddle products (rotate1) are 1 % of that.
+// from 163.7 to 113.4 ms.  Unpacked twiddle products (rotate1) are 1 % of that.
 template <bool QUAD, bool DENSE>
 __global__ void __launch_bounds__(FT, 1) k_corr_fft(const __grid_constant__ FftParams p, uint32_t total)
 {
@@ -1047,8 +1069,8 @@ __global__ void __launch_bounds__(FT, 1) k_corr_fft(const __grid_constant__ FftP
             const float2 t = r ? cmul(base_t, root32(r)) : base_t;          // e^{2 pi i n / 8192}
             float2 pr, pi, qr, qi;          // (Z[n], Z[4096 - n]) and (Z[8192 - n], Z[4096 + n])
             if (!QUAD) {
-                const cpk xk = unpack4(__ldg(X + 2 * r * GT + j)), xq = unpack4(__ldg(X + (2 * r + 1) * GT + j));
-                const cpk hk = unpack4(h[2 * r * GT + j]), hq = unpack4(h[(2 * r + 1) * GT + j]);
+                const cpk xk = unpack4(__ldg(X + 2 * r * GT + tg)), xq = unpack4(__ldg(X + (2 * r + 1) * GT + tg));
+                const cpk hk = unpack4(h[2 * r * GT + tg]), hq = unpack4(h[(2 * r + 1) * GT + tg]);
                 const float2 wr = make_float2(w.x, w.y), wi = make_float2(w.y, w.x);     // lanes n, 4096 - n
                 const float2 ykr = fma2(xk.r, hk.r, mul2(xk.i, hk.i)), yki = fma2(xk.i, hk.r, neg2(mul2(xk.r, hk.i)));
                 const float2 yqr = fma2(xq.r, hq.r, mul2(xq.i, hq.i)), yqi = fma2(xq.i, hq.r, neg2(mul2(xq.r, hq.i)));
@@ -1060,8 +1082,8 @@ __global__ void __launch_bounds__(FT, 1) k_corr_fft(const __grid_constant__ FftP
                 qr = add2(ar, wbi);
                 qi = sub2(wbr, ai);
             } else {
-                const cpk x = unpack4(__ldg(X + r * GT + j));
-                const cpk ha = unpack4(h[r * GT + j]), hb = unpack4(h[FH / 2 + r * GT + j]);
+                const cpk x = unpack4(__ldg(X + r * GT + tg));
+                const cpk ha = unpack4(h[r * GT + tg]), hb = unpack4(h[FH / 2 + r * GT + tg]);
                 const float2 yar = fma2(x.r, ha.r, mul2(x.i, ha.i)), yai = fma2(x.i, ha.r, neg2(mul2(x.r, ha.i)));
                 const float2 ybr = fma2(x.r, hb.r, mul2(x.i, hb.i)), ybi = fma2(x.i, hb.r, neg2(mul2(x.r, hb.i)));
                 // Z = Ya + i Yb, Z[N - k] = conj(Ya) + i conj(Yb)
@@ -1169,7 +1191,7 @@ __global__ void __launch_bounds__(FT, 1) k_corr_fft(const __grid_constant__ FftP
         // zero past the segment's end
         auto norms = [&](int q) -> float4 {
             if ((QUAD ? 2u : 4u) * GT * q >= nv) return make_float4(0.f, 0.f, 0.f, 0.f);
-            if (!QUAD) return __ldg(reinterpret_cast<const float4*>(nrm) + GT * q + tg);
+            if (!QUAD) return ldg_past_l1(reinterpret_cast<const float4*>(nrm) + GT * q + tg);
             const float2 f = __ldg(reinterpret_cast<const float2*>(nrm) + GT * q + tg);
             return make_float4(f.x, f.y, 0.f, 0.f);
         };
