@@ -564,8 +564,8 @@ def run_fft(ctx, bf, w, xs, ctrl, corr_per_step, alu, steps=3):
                          "frac": round(fft_flops / (k_ms / 1e3) / 1e12 / alu["fp32_tflops"], 4),
                          "peak_source": "measured FP32 FMA rate (alu_peaks)",
                          "work": "5 N log2 N nominal flops per N-point complex transform",
-                         "note": "on-chip bound: the profile puts the L1 data pipe at 61 %, the FP32 "
-                                 "pipe at 53 % and issue at 50 % of their peaks; no DRAM bound"},
+                         "note": "on-chip bound: the profile puts the L1 data pipe at 62 %, the FP32 "
+                                 "pipe at 56 % and issue at 54 % of their peaks; no DRAM bound"},
             "roofline_smem": smem_roofline(n_transforms, k_ms, clocks),
             "clocks": clocks,
             "note": "FP32 complex FFTs of 8192 points carrying real segments of 16384 samples "
@@ -580,8 +580,8 @@ def run_fft(ctx, bf, w, xs, ctrl, corr_per_step, alu, steps=3):
 # correlation kernel (ncu l1tex__data_pipe_lsu_wavefronts_mem_shared.sum over
 # the transforms of the 16 s x 16,384-template case): the passes' loads and
 # stores, the template's records and the twiddles (the segment spectrum, the
-# norms and the mirrors' shuffles cross the same pipe, another 1150)
-FFT_SMEM_WAVEFRONTS = 3570
+# norms and the mirrors' shuffles cross the same pipe, another 980)
+FFT_SMEM_WAVEFRONTS = 3600
 
 
 def torch_device_index() -> int:
