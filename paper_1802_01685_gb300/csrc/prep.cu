@@ -54,7 +54,10 @@ __device__ __forceinline__ T block_sum(T v, T* sh)
     return tot;
 }
 
-// exclusive scan over the block's threads
+// exclusive scan over the block's threads.  A thread's result holds only the
+// threads before it: taking its own part off an inclusive total would leave that
+// part's rounding in it, and S[t] must not depend on x[t ..] (quiet data before
+// loud data).
 template <typename T>
 __device__ __forceinline__ T block_excl_scan(T v, T* sh)
 {
@@ -66,13 +69,15 @@ __device__ __forceinline__ T block_excl_scan(T v, T* sh)
         if (lane >= o) inc += t;
     }
     if (lane == 31) sh[wid] = inc;
+    T ex = __shfl_up_sync(0xffffffffu, inc, 1);
+    if (lane == 0) ex = T(0);
     __syncthreads();
     T base = T(0);
 #pragma unroll
     for (int w = 0; w < SCAN_T / 32; ++w)
         if (w < wid) base += sh[w];
     __syncthreads();
-    return base + (inc - v);
+    return base + ex;
 }
 
 __device__ __forceinline__ uint32_t* block_counts(double* bsum, uint64_t nb) { return reinterpret_cast<uint32_t*>(bsum + nb); }
