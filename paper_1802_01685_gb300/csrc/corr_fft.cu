@@ -1245,28 +1245,30 @@ __global__ void __launch_bounds__(FT, 1) k_corr_fft(const __grid_constant__ FftP
             });
         // only a warp whose largest |rho| reaches its running max (ties
         // included: an earlier lag wins them) or the tail threshold looks at
-        // single lags
+        // single lags.  A NaN (finite samples that overflow the transform) counts as
+        // larger than any |rho|, as its bits do; fmaxf drops it, the squares do not.
+        float sum = pa.x + pa.y;                          // 64 terms of a thread
+        if (!(sum == sum)) m = __int_as_float(0x7fc00000);
         m = warp_max_abs(m);
         __syncwarp();
         const float best_v = __uint_as_float((uint32_t)(acc.best >> 32));
-        if (m >= fminf(thr, best_v)) {
-            if (m >= best_v) {
-                // the earliest lag that has it (a padded lag has rho = 0 and a
-                // later lag than the segment's: it cannot win)
+        if (!(m < fminf(thr, best_v))) {
+            if (!(m < best_v)) {
+                // the earliest lag that has it (a padded lag has rho = 0 and is
+                // later than the segment's), for a NaN the warp's earliest
                 uint32_t first = 0xffffffffu;
                 each([&](uint32_t t, float r) {
-                    if (fabsf(r) == m) first = min(first, t);
+                    if (!(fabsf(r) < m)) first = min(first, t);
                 });
                 first = __reduce_min_sync(0xffffffffu, first);
                 const unsigned long long key = pack_max(m, t0 + first);
-                if (lane == 0 && key > acc.best) acc.best = key;
+                if (lane == 0 && first < nv && key > acc.best) acc.best = key;
             }
-            if (m >= thr)
+            if (!(m < thr))
                 each([&](uint32_t t, float r) {
                     if (t < nv && fabsf(r) >= thr) push_tail(p, S.series_id, QUAD ? k >> 1 : k, t0 + t, r);
                 });
         }
-        float sum = pa.x + pa.y;                          // 64 terms of a thread, then 32 threads
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
         if (lane == 0) acc.ss += (double)sum;
