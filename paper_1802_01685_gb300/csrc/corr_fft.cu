@@ -82,8 +82,9 @@ static_assert(FFT_SMEM % 16 == 0 && (FFT_SMEM + ZPAD * sizeof(float2)) % 16 == 0
 constexpr int GT = FT / 2;
 constexpr int ZROW = 17, ZBLK = 16 * ZROW, ZG = 16 * ZBLK;
 constexpr int TWC_N = 6 * 256 + 15 * 16 + 2 * 256;          // float2 entries, after the TW_N of the forward transforms
-// 2 x 9: column 0; the warps' reductions; two mbarriers
-constexpr size_t CORR_SMEM = (size_t)(2 * ZG + FH + TWC_N / 2 + 2 * 9 + FT / 32 + 1) * sizeof(float4);
+// 2 x 9: column 0; the warps' max keys; two mbarriers; the threads' sums
+constexpr int CORR_ACC = 2 * ZG + FH + TWC_N / 2 + 2 * 9;
+constexpr size_t CORR_SMEM = (size_t)(CORR_ACC + FT / 32 + 1 + FT / 2) * sizeof(float4);
 static_assert(CORR_SMEM <= 227 * 1024, "the correlation kernel fits one SM's shared memory");
 static_assert(TW_N % 2 == 0 && TWC_N % 2 == 0, "16-byte tables");
 
@@ -876,6 +877,16 @@ __device__ __forceinline__ void mbar_wait(uint64_t* bar, uint32_t parity, int* e
     if (err) atomicCAS(err, DEV_OK, DEV_TIMEOUT_FFT);
 }
 
+// s.x + s.y += a, s.x rounded and s.y what the roundings left (Knuth's two-sum): the
+// sum of rho^2 to 48 bits without FP64's pipe, whose conversions and additions made
+// the GW step 115.6 ms instead of 113.0 (light curves 29.2, 28.5)
+__device__ __forceinline__ void add_exact(float2& s, float a)
+{
+    const float h = __fadd_rn(s.x, a), b = __fsub_rn(h, s.x);
+    s.y = __fadd_rn(s.y, __fadd_rn(__fsub_rn(s.x, __fsub_rn(h, b)), __fsub_rn(a, b)));
+    s.x = h;
+}
+
 // 16 bytes of global memory past L1: the norms, which would displace the segment
 // spectra there (light curves 8.43 -> 8.27 ms, a 16 s plan 529 -> 526 us, the 64 s
 // step 7.32 -> 7.38 ms; the spectra themselves past L1 cost 4 % there)
@@ -949,14 +960,11 @@ __global__ void __launch_bounds__(FT, 1) k_corr_fft(const __grid_constant__ FftP
     const float2* const twb = twa + 6 * GT;               // [15][16]
     const float4* const twp = reinterpret_cast<const float4*>(twb + 15 * 16);   // [256] pairs
     float4* const col0 = h + FH + TWC_N / 2 + 9 * g;      // column 0's inputs 2048, 2304 .. 3840, and 0
-    // the warp's reductions over the (row, series) so far, kept out of the registers:
-    // its packed max key (0: none yet; a lag below its value and the tail threshold
-    // changes nothing) and its sum of rho^2
-    struct Acc {
-        unsigned long long best;
-        double ss;
-    };
-    Acc& acc = reinterpret_cast<Acc*>(h + FH + TWC_N / 2 + 2 * 9)[threadIdx.x >> 5];
+    // the reductions over the (row, series) so far, kept out of the registers: the
+    // warp's packed max key (0: none yet; a lag below its value and the tail threshold
+    // changes nothing) and the thread's sum of rho^2, a pair of FP32 values
+    unsigned long long& best = reinterpret_cast<ulonglong2*>(h + FH + TWC_N / 2 + 2 * 9)[threadIdx.x >> 5].x;
+    float2& ss = reinterpret_cast<float2*>(h + FH + TWC_N / 2 + 2 * 9 + FT / 32 + 1)[threadIdx.x];
     // the group's mbarrier: its work array is read
     uint64_t* const zread = reinterpret_cast<uint64_t*>(h + FH + TWC_N / 2 + 2 * 9 + FT / 32) + g;
     const int BAR_G = 1 + g, BAR_EMPTY = 3, BAR_FULL = 4;          // FULL: two, by the parity of the row
@@ -1015,7 +1023,8 @@ __global__ void __launch_bounds__(FT, 1) k_corr_fft(const __grid_constant__ FftP
         (void)BF_BOUNDS(p.err, k + KR - 1 < p.k_end && k >= p.hrow0 && seg < S.nseg);
         if (fresh) {
             thr = S.sigma_pred ? S.kappa * S.sigma_pred[o] : p.thr;
-            if (lane == 0) acc = Acc{0ull, 0.0};
+            if (lane == 0) best = 0ull;
+            ss = make_float2(0.f, 0.f);
         }
         const uint32_t t0 = seg * p.V;
         const uint32_t nv = min(p.V, S.L - t0);
@@ -1243,15 +1252,21 @@ __global__ void __launch_bounds__(FT, 1) k_corr_fft(const __grid_constant__ FftP
             each([&](uint32_t t, float r) {
                 if (t < nv && BF_BOUNDS(p.err, t0 + t < S.L)) S.rho[(size_t)o * S.L + t0 + t] = r;
             });
+        {
+            float2 t = ss;                                // 32 terms each in FP32 (pair route 16)
+            add_exact(t, pa.x);
+            add_exact(t, pa.y);
+            ss = t;
+            // a NaN (finite samples that overflow the transform) counts as larger than any
+            // |rho|, as its bits do; fmaxf drops it, the squares do not
+            if (!(t.x == t.x)) m = __int_as_float(0x7fc00000);
+        }
         // only a warp whose largest |rho| reaches its running max (ties
         // included: an earlier lag wins them) or the tail threshold looks at
-        // single lags.  A NaN (finite samples that overflow the transform) counts as
-        // larger than any |rho|, as its bits do; fmaxf drops it, the squares do not.
-        float sum = pa.x + pa.y;                          // 64 terms of a thread
-        if (!(sum == sum)) m = __int_as_float(0x7fc00000);
+        // single lags
         m = warp_max_abs(m);
         __syncwarp();
-        const float best_v = __uint_as_float((uint32_t)(acc.best >> 32));
+        const float best_v = __uint_as_float((uint32_t)(best >> 32));
         if (!(m < fminf(thr, best_v))) {
             if (!(m < best_v)) {
                 // the earliest lag that has it (a padded lag has rho = 0 and is
@@ -1262,24 +1277,27 @@ __global__ void __launch_bounds__(FT, 1) k_corr_fft(const __grid_constant__ FftP
                 });
                 first = __reduce_min_sync(0xffffffffu, first);
                 const unsigned long long key = pack_max(m, t0 + first);
-                if (lane == 0 && first < nv && key > acc.best) acc.best = key;
+                if (lane == 0 && first < nv && key > best) best = key;
             }
             if (!(m < thr))
                 each([&](uint32_t t, float r) {
                     if (t < nv && fabsf(r) >= thr) push_tail(p, S.series_id, QUAD ? k >> 1 : k, t0 + t, r);
                 });
         }
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
-        if (lane == 0) acc.ss += (double)sum;
         uint32_t nrow = row;
         int ns = s;
         asm volatile("" : "+r"(seg));                     // recomputed here, not kept in registers
         advance(nrow, ns, seg);
         fresh = !more || ns != s || nrow != row;
-        if (fresh && lane == 0) {
-            atomicMax(S.vmax + o, acc.best);
-            atomicAdd(S.sumsq + o, acc.ss);
+        if (__any_sync(0xffffffffu, fresh)) {             // the whole warp's: as a vote it needs no convergence barrier
+            const float2 t = ss;
+            double sum = (double)t.x + (t.y == t.y ? (double)t.y : 0.0);     // an infinity leaves a NaN beside it
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+            if (lane == 0) {
+                atomicMax(S.vmax + o, best);
+                atomicAdd(S.sumsq + o, sum);
+            }
         }
         if (!more) break;
         // the spectra of the next item's row: fetched by this group (all its
