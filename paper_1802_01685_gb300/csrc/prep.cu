@@ -209,21 +209,27 @@ __global__ void __launch_bounds__(SCAN_T) k_prefix(const __grid_constant__ PrepB
     }
 }
 
-// 1/sqrt(nu) for nu > 0, rounded to FP32 from FP64: the FP32 value of nu's
-// mantissa with an even exponent, m in [1, 4), then one Newton step
-// y += y (1 - m y^2) / 2 in FP64 (relative error 3/8 (2 * 2^-22)^2, far inside
-// FP32's half ulp), scaled back exactly.  Energies outside 2^+-240 (the result
-// would leave the range of normal floats) take the FP64 root and division.
+// 1/sqrt(m) for m in [1, 4) in FP64: from FP32's value y with h = 1 - m y^2, which
+// is rounded once (y^2 is exact), y (1 - h)^(-1/2) = y (1 + h/2 + 3 h^2/8 + ...).
+// |h| <= 2^-20, so the series ends below 2^-61 of the value: closer than the
+// FP64 root and division that it stands for, in five instructions of the slow pipe.
+__device__ __forceinline__ double inv_root(double m)
+{
+    const double y = (double)rsqrtf((float)m);
+    const double h = fma(-m, y * y, 1.0);
+    return fma(y, h * fma(0.375, h, 0.5), y);
+}
+
+// 1/sqrt(nu) for nu > 0, rounded to FP32 from FP64: of nu's mantissa with an even
+// exponent, scaled back exactly.  Energies outside 2^+-240 (the result would leave
+// the range of normal floats) take the FP64 root and division.
 __device__ __forceinline__ float inv_sqrt(double nu)
 {
     const int hi = __double2hiint(nu);
     const int e = ((hi >> 20) - 1023) & ~1;               // even exponent
     if (e < -240 || e > 240) return (float)(1.0 / sqrt(nu));
     const double m = __hiloint2double(hi - (e << 20), __double2loint(nu));
-    const double y = (double)rsqrtf((float)m);
-    const double h = fma(-m * y, y, 1.0);                 // 1 - m y^2
-    const float r = (float)fma(0.5 * y, h, y);
-    return r * __int_as_float((127 - e / 2) << 23);       // 2^(-e/2)
+    return (float)inv_root(m) * __int_as_float((127 - e / 2) << 23);       // 2^(-e/2)
 }
 
 // Norms and split rows of series blockIdx.y, one index per thread.
