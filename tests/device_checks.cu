@@ -1,8 +1,13 @@
 // Checks of device functions that no call of the library shows by itself.  The
 // sources are included, so that the functions tested are the library's.
+#include <algorithm>
 #include <cstdio>
+#include <cstring>
+#include <numeric>
 
 #include "prep.cu"
+#include "permute.cu"
+#include "corr_common.cuh"
 
 namespace bfi {
 std::atomic<uint64_t> g_launches{0};
@@ -18,15 +23,6 @@ using namespace bfi;
             return 2;                                                             \
         }                                                                         \
     } while (0)
-
-// a counter-based draw (the splitmix64 finaliser)
-__device__ uint64_t splitmix64(uint64_t z)
-{
-    z += 0x9E3779B97F4A7C15ull;
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
-}
 
 // mantissas of window energies in [1, 4): the largest relative distance of the
 // library's 1 / sqrt from FP64's, in units of 2^-53; and the norms of energies
@@ -60,4 +56,53 @@ static int norms()
     return 0;
 }
 
-int main() { return norms(); }
+// The control's four steps with 2^bits buckets for n samples, so few that every
+// bucket reaches past a block's neighbourhood, against a stable sort by key.
+static int crowded(uint32_t n, int bits, uint64_t seed)
+{
+    auto mix = [](uint64_t z) {
+        z += 0x9E3779B97F4A7C15ull;
+        z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+        z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+        return z ^ (z >> 31);
+    };
+    std::vector<float> x(n), got(n);
+    std::iota(x.begin(), x.end(), 0.f);
+    std::vector<uint32_t> want(n);
+    std::iota(want.begin(), want.end(), 0u);
+    std::stable_sort(want.begin(), want.end(),
+                     [&](uint32_t a, uint32_t b) { return mix(seed ^ a) < mix(seed ^ b); });
+    const uint32_t B = 1u << bits;
+    const int shift = 64 - bits;
+    float *in = nullptr, *out = nullptr;
+    uint32_t* s = nullptr;
+    CK(cudaMalloc(&in, n * 4));
+    CK(cudaMalloc(&out, n * 4));
+    CK(cudaMalloc(&s, (2 * (size_t)B + 2 * (size_t)n) * 4));
+    uint32_t *count = s, *begin = s + B, *slot = begin + B, *idx = slot + n;
+    CK(cudaMemcpy(in, x.data(), n * 4, cudaMemcpyHostToDevice));
+    CK(cudaMemset(out, 0xff, n * 4));
+    CK(cudaMemset(count, 0, B * 4));
+    const unsigned grid = (n + SORT_T - 1) / SORT_T;
+    k_perm_count<<<grid, SORT_T>>>(n, seed, shift, count, slot);
+    k_perm_scan<<<(B + SCAN_TILE - 1) / SCAN_TILE, SCAN_THREADS>>>(count, B, begin);
+    k_perm_scatter<<<grid, SORT_T>>>(n, seed, shift, begin, slot, idx);
+    k_perm_rank<<<grid, SORT_T>>>(in, n, seed, shift, begin, count, idx, out);
+    CK(cudaGetLastError());
+    CK(cudaMemcpy(got.data(), out, n * 4, cudaMemcpyDeviceToHost));
+    uint32_t wrong = 0;
+    for (uint32_t j = 0; j < n; ++j) wrong += got[j] != (float)want[j] ? 1u : 0u;
+    printf("crowded_wrong %u %d %u\n", n, bits, wrong);
+    cudaFree(in);
+    cudaFree(out);
+    cudaFree(s);
+    return 0;
+}
+
+int main()
+{
+    int rc = norms();
+    for (uint32_t n : {257u, 5000u, 20001u})
+        for (int bits : {2, 4, 6}) rc = rc ? rc : crowded(n, bits, 0x1234567ull + n);
+    return rc;
+}

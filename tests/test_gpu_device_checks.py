@@ -1,5 +1,6 @@
 """Device functions that no call of the library shows by themselves, through
-device_checks.cu: the inverse window norm over its whole range."""
+device_checks.cu: the inverse window norm over its whole range, and the
+control's rank step for buckets far more crowded than uniform keys make them."""
 import os
 import subprocess
 
@@ -30,3 +31,8 @@ def test_inverse_norm_is_fp64s(lines):
     taken four times."""
     (_, worst, wrong), = [a for a in lines if a[0] == "norms"]
     assert float(worst) <= 3.0 and int(wrong) <= 8, (worst, wrong)
+
+
+def test_crowded_buckets(lines):
+    got = [a for a in lines if a[0] == "crowded_wrong"]
+    assert len(got) == 9 and all(int(a[3]) == 0 for a in got), got
