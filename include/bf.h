@@ -601,10 +601,10 @@ const char* bf_last_error(void);
 const char* bf_status_string(bf_status s);
 int bf_abi_version(void);
 
-/* Self-test of the bounded waits that guard the tensor-core kernel's
- * pipeline (every mbarrier wait gives up after a time limit, records a code
- * in the context's device status word and lets the kernel drain and return,
- * so that no wait can hang the GPU).  Runs the same wait on an mbarrier that
+/* Self-test of the bounded waits that guard the pipelines of the tensor-core
+ * and FFT kernels (every mbarrier wait gives up after a time limit, records a
+ * code in the device status word and lets the kernel drain and return, so
+ * that no wait can hang the GPU).  Runs the same wait on an mbarrier that
  * receives its one arrival when `signal` is nonzero and never otherwise, with
  * a limit of limit_us microseconds (at most 1,000,000), synchronously on the
  * context stream.  Returns BF_OK when the arrival came, BF_EDEVICE when the

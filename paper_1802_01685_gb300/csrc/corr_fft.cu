@@ -82,9 +82,9 @@ static_assert(FFT_SMEM % 16 == 0 && (FFT_SMEM + ZPAD * sizeof(float2)) % 16 == 0
 constexpr int GT = FT / 2;
 constexpr int ZROW = 17, ZBLK = 16 * ZROW, ZG = 16 * ZBLK;
 constexpr int TWC_N = 6 * 256 + 15 * 16 + 2 * 256;          // float2 entries, after the TW_N of the forward transforms
-// 2 x 9: column 0; the warps' max keys; two mbarriers; the threads' sums
+// 2 x 9: column 0; the warps' max keys; two mbarriers; the threads' sums; the abort flag
 constexpr int CORR_ACC = 2 * ZG + FH + TWC_N / 2 + 2 * 9;
-constexpr size_t CORR_SMEM = (size_t)(CORR_ACC + FT / 32 + 1 + FT / 2) * sizeof(float4);
+constexpr size_t CORR_SMEM = (size_t)(CORR_ACC + FT / 64 + 1 + FT / 2 + 1) * sizeof(float4);
 static_assert(CORR_SMEM <= 227 * 1024, "the correlation kernel fits one SM's shared memory");
 static_assert(TW_N % 2 == 0 && TWC_N % 2 == 0, "16-byte tables");
 
@@ -846,35 +846,19 @@ __device__ __forceinline__ void bar_arrive(int id, int count)
 
 // A work array's mbarrier, of one phase a transform: the group's warps arrive
 // when they have read their last of the transform from it, and wait for all
-// before they write the next one's.  The wait is bounded (seconds, against the
-// microseconds that it takes); on expiry the status word is set and the kernel
-// goes on, so that it ends.
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"((unsigned)__cvta_generic_to_shared(bar)), "r"(count)
-                 : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar)
+// before they write the next one's.  On expiry of the wait the status word is set
+// and the kernel goes on without any further wait on these mbarriers, so that it
+// ends (its outputs are not given out).
+__device__ __forceinline__ void warp_arrive(uint32_t bar)
 {
     __syncwarp();
-    if ((threadIdx.x & 31) == 0)
-        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"((unsigned)__cvta_generic_to_shared(bar))
-                     : "memory");
+    if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
 }
-__device__ __forceinline__ void mbar_wait(uint64_t* bar, uint32_t parity, int* err)
+__device__ __forceinline__ void work_array_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err)
 {
-    const unsigned a = (unsigned)__cvta_generic_to_shared(bar);
-    for (int n = 0; n < (1 << 22); ++n) {
-        uint32_t done;
-        asm volatile("{\n\t.reg .pred p;\n\t"
-                     "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-                     "selp.u32 %0, 1, 0, p;\n\t}"
-                     : "=r"(done)
-                     : "r"(a), "r"(parity)
-                     : "memory");
-        if (done) return;
-    }
-    if (err) atomicCAS(err, DEV_OK, DEV_TIMEOUT_FFT);
+    if (mbar_try_wait(bar, parity) || *abort_flag || mbar_wait(bar, parity, abort_flag)) return;
+    if (err && !*abort_flag) record_error(err, DEV_TIMEOUT_FFT);
+    *abort_flag = 1;
 }
 
 // s.x + s.y += a, s.x rounded and s.y what the roundings left (Knuth's two-sum): the
@@ -963,10 +947,11 @@ __global__ void __launch_bounds__(FT, 1) k_corr_fft(const __grid_constant__ FftP
     // the reductions over the (row, series) so far, kept out of the registers: the
     // warp's packed max key (0: none yet; a lag below its value and the tail threshold
     // changes nothing) and the thread's sum of rho^2, a pair of FP32 values
-    unsigned long long& best = reinterpret_cast<ulonglong2*>(h + FH + TWC_N / 2 + 2 * 9)[threadIdx.x >> 5].x;
-    float2& ss = reinterpret_cast<float2*>(h + FH + TWC_N / 2 + 2 * 9 + FT / 32 + 1)[threadIdx.x];
+    unsigned long long& best = reinterpret_cast<unsigned long long*>(csm + CORR_ACC)[threadIdx.x >> 5];
+    float2& ss = reinterpret_cast<float2*>(csm + CORR_ACC + FT / 64 + 1)[threadIdx.x];
     // the group's mbarrier: its work array is read
-    uint64_t* const zread = reinterpret_cast<uint64_t*>(h + FH + TWC_N / 2 + 2 * 9 + FT / 32) + g;
+    const uint32_t zread = smem_u32(csm + CORR_ACC + FT / 64) + 8 * g;
+    volatile int* const abort_flag = reinterpret_cast<volatile int*>(csm + CORR_ACC + FT / 64 + 1 + FT / 2);
     const int BAR_G = 1 + g, BAR_EMPTY = 3, BAR_FULL = 4;          // FULL: two, by the parity of the row
     constexpr uint32_t BINS = QUAD ? FH : FN;             // complex bins per segment
     constexpr uint32_t KR = QUAD ? 2 : 1;                 // template rows per item
@@ -982,6 +967,7 @@ __global__ void __launch_bounds__(FT, 1) k_corr_fft(const __grid_constant__ FftP
         return reinterpret_cast<const float4*>(p.hspec + (size_t)(p.k_lo + row * KR - p.hrow0) * BINS);
     };
     if (tg == 0) mbar_init(zread, GT / 32);
+    if (threadIdx.x == 0) *abort_flag = 0;
     {
         const float4* src = reinterpret_cast<const float4*>(p.tw + TW_N);
         for (int e = threadIdx.x; e < TWC_N / 2; e += FT) cp_async16(h + FH + e, src + e);
@@ -1143,7 +1129,7 @@ __global__ void __launch_bounds__(FT, 1) k_corr_fft(const __grid_constant__ FftP
         }
         // every warp has read the transform before (item / 2 of them) from the work
         // array; asked for here, ahead of the arithmetic, and not at the writes (1 %)
-        mbar_wait(zread, ((item >> 1) & 1) ^ 1, p.err);
+        work_array_wait(zread, ((item >> 1) & 1) ^ 1, abort_flag, p.err);
         __syncwarp();
         // pass 1: out k0 = q at position 4 k1 + k2 of dft16, q = k1 + 4 k2; twiddle e^{2 pi i q j / 4096}
         dft16_pk(v);
@@ -1194,7 +1180,7 @@ __global__ void __launch_bounds__(FT, 1) k_corr_fft(const __grid_constant__ FftP
 #pragma unroll
             for (int r = 0; r < 16; ++r) v[r] = unpack4(zz[r]);
         }
-        mbar_arrive(zread);
+        warp_arrive(zread);
         // norms of the lags of this thread's output q: lags 4 k .. 4 k + 3 in the order
         // 0, 2, 1, 3 (real route), lags 2 k, 2 k + 1 (pair route), stored by (q, tg);
         // zero past the segment's end

@@ -68,7 +68,6 @@ struct Geo {
 };
 static_assert(Geo<512>::STAGE_BYTES == 51200, "stage layout");
 static_assert(Geo<512>::SMEM <= 232448 && Geo<256>::SMEM <= 232448, "shared memory per CTA");
-constexpr uint64_t TIMEOUT_NS = 10ull * 1000 * 1000 * 1000;
 constexpr uint32_t TMEM_COLS = 512;
 
 // instruction descriptors, kind::f16, D = F32, both operands K-major, N = 256,
@@ -78,61 +77,10 @@ constexpr uint32_t IDESC_BF16 = (1u << 4) | (1u << 7) | (1u << 10) | ((256u >> 3
                                 ((128u >> 4) << 24);
 constexpr uint32_t IDESC_F16 = (1u << 4) | ((256u >> 3) << 17) | ((128u >> 4) << 24);
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p)
-{
-    return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ uint64_t globaltimer()
-{
-    uint64_t t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes)
 {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
                  : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(uint32_t bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-// Bounded wait.  Returns false on timeout or when another role aborted.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity,
-                                          volatile int* abort_flag, bool honour_abort = true,
-                                          uint64_t limit_ns = TIMEOUT_NS)
-{
-    if (mbar_try_wait(bar, parity)) return true;
-    const uint64_t t0 = globaltimer();
-    for (uint32_t it = 1;; ++it) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if ((it & 63) == 0) {
-            if (honour_abort && *abort_flag) return false;
-            if (globaltimer() - t0 > limit_ns) return false;
-        }
-    }
 }
 
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes,
@@ -354,11 +302,6 @@ __device__ __forceinline__ void epi_tails_quad(const float (&q)[16], const float
         const float v = q[j] * inv[cb + j];
         if (cb + j < nvalid && v >= thr) push_candidate(p, series, chirp, lag0 + cb + j, v);
     }
-}
-
-__device__ __forceinline__ void record_error(int* err, int code)
-{
-    atomicCAS(err, 0, code);
 }
 
 struct TileCoord {

@@ -99,9 +99,41 @@ static int crowded(uint32_t n, int bits, uint64_t seed)
     return 0;
 }
 
+// The wait that both correlation kernels use, on an mbarrier that nothing arrives
+// at: with a limit of 20 ms, then with the abort flag set.
+__global__ void k_wait_check(unsigned long long* ns, int* ok)
+{
+    __shared__ __align__(8) uint64_t bar;
+    __shared__ int abort_word;
+    if (threadIdx.x != 0) return;
+    mbar_init(smem_u32(&bar), 1);
+    abort_word = 0;
+    for (int i = 0; i < 2; ++i) {
+        const uint64_t t0 = globaltimer();
+        ok[i] = mbar_wait(smem_u32(&bar), 0, &abort_word, true, i ? 1000000000ull : 20000000ull) ? 1 : 0;
+        ns[i] = globaltimer() - t0;
+        abort_word = 1;
+    }
+}
+
+static int waits()
+{
+    unsigned long long *d = nullptr, h[2];
+    int *o = nullptr, ok[2];
+    CK(cudaMalloc(&d, sizeof h));
+    CK(cudaMalloc(&o, sizeof ok));
+    k_wait_check<<<1, 32>>>(d, o);
+    CK(cudaGetLastError());
+    CK(cudaMemcpy(h, d, sizeof h, cudaMemcpyDeviceToHost));
+    CK(cudaMemcpy(ok, o, sizeof ok, cudaMemcpyDeviceToHost));
+    printf("wait %llu %d %llu %d\n", h[0], ok[0], h[1], ok[1]);
+    return 0;
+}
+
 int main()
 {
     int rc = norms();
+    rc = rc ? rc : waits();
     for (uint32_t n : {257u, 5000u, 20001u})
         for (int bits : {2, 4, 6}) rc = rc ? rc : crowded(n, bits, 0x1234567ull + n);
     return rc;

@@ -1,6 +1,7 @@
 """Device functions that no call of the library shows by themselves, through
-device_checks.cu: the inverse window norm over its whole range, and the
-control's rank step for buckets far more crowded than uniform keys make them."""
+device_checks.cu: the inverse window norm over its whole range, the bounded
+wait of the correlation kernels, and the control's rank step for buckets far more
+crowded than uniform keys make them."""
 import os
 import subprocess
 
@@ -31,6 +32,14 @@ def test_inverse_norm_is_fp64s(lines):
     taken four times."""
     (_, worst, wrong), = [a for a in lines if a[0] == "norms"]
     assert float(worst) <= 3.0 and int(wrong) <= 8, (worst, wrong)
+
+
+def test_wait_is_bounded_in_time(lines):
+    """It ends at its limit, by the clock and not by a count of tries, and soon
+    once another wait of the block has run out (64 tries)."""
+    (_, ns, ok, ns_abort, ok_abort), = [a for a in lines if a[0] == "wait"]
+    assert int(ok) == 0 and 20_000_000 <= int(ns) < 500_000_000, ns
+    assert int(ok_abort) == 0 and int(ns_abort) < 500_000_000, ns_abort
 
 
 def test_crowded_buckets(lines):
