@@ -562,7 +562,9 @@ bf_status bf_control_randomize_static(const float* in, size_t n, uint64_t seed, 
  * of template spectra on the FFT route, counted against the budget), refilled
  * every iteration with what that iteration correlates.  BF_EAGAIN: queue
  * full.  BF_ENOMEM: the request alone exceeds the budget.  BF_EINVAL: bad
- * request.
+ * request.  A kernel that reports an internal timeout fails every request that
+ * is active then, with BF_EDEVICE from bf_serve_poll; requests and calls on
+ * the context do not share a status word.
  */
 typedef struct {
     const float* series;     /* host or device, n samples                        */
@@ -612,6 +614,13 @@ int bf_abi_version(void);
  * usable), BF_EINVAL for a limit out of range.  *waited_us (if not NULL) gets
  * the time the wait took. */
 bf_status bf_selftest_wait(bf_ctx* ctx, int signal, uint32_t limit_us, double* waited_us);
+/* The same for the serving loop: before its next iteration that has an active
+ * request the loop launches one such wait, which nothing ends but its limit.  A
+ * kernel serves several requests and cannot say which it left unfinished, so
+ * every request active then fails with BF_EDEVICE; those submitted later are
+ * served.  Returns at once.  BF_EINVAL for a limit out of range or before the
+ * first bf_serve_submit. */
+bf_status bf_selftest_serve(bf_ctx* ctx, uint32_t limit_us);
 /* Number of kernels this library has launched in the process so far (all
  * contexts); a diagnostic for benchmarks.  The paper has no counterpart. */
 uint64_t bf_kernel_launches(void);

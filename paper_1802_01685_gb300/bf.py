@@ -162,6 +162,7 @@ def load() -> C.CDLL:
             "bf_status_string": (C.c_char_p, [i]),
             "bf_abi_version": (i, []),
             "bf_selftest_wait": (i, [p, i, C.c_uint32, P(d)]),
+            "bf_selftest_serve": (i, [p, C.c_uint32]),
             "bf_kernel_launches": (u64, []),
             "bf_probe_alu_peaks": (i, [i, P(d), P(d)]),
         }
@@ -573,6 +574,12 @@ def bf_selftest_wait(ctx: int, signal: bool, limit_us: int) -> float:
     w = C.c_double()
     _check(load().bf_selftest_wait(ctx, int(bool(signal)), int(limit_us), C.byref(w)))
     return w.value
+
+
+def bf_selftest_serve(ctx: int, limit_us: int) -> None:
+    """Lets one unsignalled wait run out on the serving stream: every request
+    active then fails with BF_EDEVICE."""
+    _check(load().bf_selftest_serve(ctx, int(limit_us)))
 
 
 def bf_abi_version() -> int:

@@ -469,7 +469,7 @@ static uint64_t whole_tiles(uint64_t tiles, uint32_t M_pad, int n_sm)
 
 cudaError_t launch_segments(bf_ctx* ctx, const std::vector<Seg>& segs, int precision, float thr,
                             Candidate* cand, unsigned int* cand_count, unsigned int cand_cap,
-                            cudaStream_t st, uint64_t* tiles_out, int lt)
+                            cudaStream_t st, uint64_t* tiles_out, int lt, int* err)
 {
     if (precision != BF_FP32 && lt == 0 && !segs.empty()) lt = choose_lag_tile(ctx, segs[0], precision, st);
     if (precision == BF_FP32) lt = SIMT_TILE_L;
@@ -489,7 +489,7 @@ cudaError_t launch_segments(bf_ctx* ctx, const std::vector<Seg>& segs, int preci
         p.cand = cand;
         p.cand_count = cand_count;
         p.cand_cap = cand_cap;
-        p.err = ctx->d_err;
+        p.err = err ? err : ctx->d_err;
         p.idesc = tc_idesc(precision);
         // accumulator chunks of 2048 samples (split-BF16) or 1024 (split-FP16)
         p.kchunk_log2 = precision == BF_SPLIT_FP16 ? 4u : 5u;
@@ -609,6 +609,7 @@ bf_status alloc_result(bf_ctx* ctx, const bf_bank* bank, const bf_opts& o,
 {
     std::unique_ptr<bf_result> r(new bf_result());
     r->ctx = ctx;
+    r->err = ctx->d_err;
     r->n_series = lengths.size();
     r->K = o.bank_end - o.bank_begin;
     r->k_begin = o.bank_begin;
@@ -745,7 +746,7 @@ bf_status finalize_result(bf_ctx* ctx, const bf_bank* bank, bf_result* r, cudaSt
         FinalizeParams fp{};
         fp.s0 = (uint32_t)s0;
         fp.n_chirps = (uint32_t)bank->K;
-        fp.err = ctx->d_err;
+        fp.err = r->err;
         fp.n = (uint32_t)std::min(S - s0, (size_t)MAX_FIN);
         for (uint32_t i = 0; i < fp.n; ++i) {
             const size_t s = s0 + i;
@@ -777,7 +778,7 @@ bf_status finalize_result(bf_ctx* ctx, const bf_bank* bank, bf_result* r, cudaSt
         p.n_series = (uint32_t)S;
         p.K = (uint32_t)K;
         p.head = r->host;
-        p.err = ctx->d_err;
+        p.err = r->err;
         p.counts = r->cand_count;
         if (r->host_data) {
             p.h_mean = r->host_mean();
@@ -970,15 +971,12 @@ static bf_status status_of(unsigned int w)
     return BF_OK;
 }
 
-static bf_status device_status_of(bf_ctx* ctx, int h)
+static bf_status device_status_of(int h)
 {
-    if (h != DEV_OK) {
-        cudaMemset(ctx->d_err, 0, sizeof(int));
-        if (h == DEV_BOUNDS) set_error("a kernel's bounds check failed (debug build)");
-        else set_error("kernel reported internal timeout (code %d)", h);
-        return BF_EDEVICE;
-    }
-    return BF_OK;
+    if (h == DEV_OK) return BF_OK;
+    if (h == DEV_BOUNDS) set_error("a kernel's bounds check failed (debug build)");
+    else set_error("kernel aborted after a timeout (status word %d)", h);
+    return BF_EDEVICE;
 }
 
 bf_status result_status(const bf_result* r)
@@ -989,25 +987,31 @@ bf_status result_status(const bf_result* r)
     return status_of(w);
 }
 
+// reads the context's word, and clears it where it held a code
 bf_status check_device_status(bf_ctx* ctx)
 {
     int h = 0;
     cudaError_t e = cudaMemcpy(&h, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess && h != DEV_OK) e = cudaMemset(ctx->d_err, 0, sizeof(int));
     if (e != cudaSuccess) return cuda_fail(e, "reading kernel status");
-    return device_status_of(ctx, h);
+    return device_status_of(h);
 }
 
-bf_status result_complete(bf_result* r)
+bf_status result_complete(bf_result* r, bool* kernel_failed)
 {
     HostHead h{};
     if (r->host) {
         h = *r->host;
     } else {
-        cudaError_t e = cudaMemcpy(&h.err, r->ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost);
+        cudaError_t e = cudaMemcpy(&h.err, r->err, sizeof(int), cudaMemcpyDeviceToHost);
         if (e == cudaSuccess) e = cudaMemcpy(&h.cand_count, r->cand_count, 2 * sizeof(unsigned int), cudaMemcpyDeviceToHost);
         if (e != cudaSuccess) return cuda_fail(e, "reading the search's status");
     }
-    bf_status st = device_status_of(r->ctx, h.err);
+    if (kernel_failed) *kernel_failed = h.err != DEV_OK;
+    // what the result holds is a copy taken when it was finished: the context's
+    // word is cleared as it stands now (the serving loop clears its own)
+    if (h.err != DEV_OK && r->err == r->ctx->d_err) check_device_status(r->ctx);
+    bf_status st = device_status_of(h.err);
     if (st == BF_OK) st = check_canaries(r);        // debug builds: no output written past its end
     if (st == BF_OK) st = status_of(h.status);      // every sample must be finite
     if (st != BF_OK) return st;

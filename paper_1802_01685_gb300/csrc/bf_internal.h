@@ -44,7 +44,8 @@ constexpr int K_ALIGN = 128;              // bank size padded to this
 constexpr int MAX_SEG = 64;               // series (segments) per launch
 constexpr uint32_t TILE_BYTES_A = TC_TILE_T * TC_BK * 2;   // 16 KiB per k-block
 
-// device error codes written to the context's status word
+// device error codes written to a status word: the context's for calls and plans,
+// the serving loop's own for what it launches
 enum : int { DEV_OK = 0, DEV_TIMEOUT_FULL = 1, DEV_TIMEOUT_EMPTY = 2,
              DEV_TIMEOUT_TMEM = 3, DEV_TMEM_ALLOC = 4, DEV_BOUNDS = 5,
              DEV_TIMEOUT_FFT = 6 };
@@ -52,7 +53,7 @@ enum : int { DEV_OK = 0, DEV_TIMEOUT_FULL = 1, DEV_TIMEOUT_EMPTY = 2,
 // Debug builds (-DBF_DEBUG_BOUNDS, built as libbf_debug.so): the kernels
 // check the indices their outputs, staging buffers and tables rely on --
 // invariants that the launch set-up guarantees, so a release build does not
-// test them.  A failed check records DEV_BOUNDS in the context's status word
+// test them.  A failed check records DEV_BOUNDS in the status word
 // (the first code recorded stays) and skips the access; the call then
 // returns BF_EDEVICE.  Nothing traps.  In release builds BF_BOUNDS is `true`.
 #ifdef BF_DEBUG_BOUNDS
@@ -323,7 +324,7 @@ struct FinalizeSeries {
 // and into the result's host copy (mapped page-locked memory; head may be
 // nullptr) the status words, the mean and the histograms.
 struct HostHead {
-    int err;                        // the context's status word
+    int err;                        // the kernels' status word
     unsigned int cand_count;
     unsigned int status;            // bit 0: a series holds a non-finite sample
 };
@@ -517,6 +518,9 @@ struct bf_result {
     // device word after cand_count, zeroed with it: bit 0 is set by the series
     // preparation when a series holds a non-finite sample
     unsigned int* status = nullptr;
+    // the status word of the kernels that make this result: the context's, or the
+    // serving loop's
+    int* err = nullptr;
     // Host copy, written by the finalize kernels: the head, and with host_data
     // also max, argmax and sigma [S][K], the histograms [S][nbins] and the mean
     // [K].  host_ready: the work that wrote it has completed.

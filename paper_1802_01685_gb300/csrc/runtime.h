@@ -65,10 +65,11 @@ Seg make_segment(const PreparedSeries& ps, uint32_t series_id, const bf_bank* ba
                  size_t k_end, uint32_t tt_first, uint32_t tt_count, int precision,
                  unsigned long long* packed_s, double* sumsq_s, float* rho = nullptr);
 
-// lt: lags per tensor-core tile (256 or 512), 0 = autotuned; ignored by FP32
+// lt: lags per tensor-core tile (256 or 512), 0 = autotuned; ignored by FP32.
+// err: the status word of the launch (nullptr: the context's)
 cudaError_t launch_segments(bf_ctx* ctx, const std::vector<Seg>& segs, int precision, float thr,
                             Candidate* cand, unsigned int* cand_count, unsigned int cand_cap,
-                            cudaStream_t st, uint64_t* tiles_out, int lt = 0);
+                            cudaStream_t st, uint64_t* tiles_out, int lt = 0, int* err = nullptr);
 // The autotuner: lags per tile for this precision and template length, timed
 // once per context on a synthetic problem over the segment's template tiles.
 int choose_lag_tile(bf_ctx* ctx, const Seg& g, int precision, cudaStream_t st);
@@ -90,7 +91,8 @@ bf_status check_canaries(const bf_result* r);
 
 // the status of a search whose work has completed (BF_EDEVICE, BF_EINVAL for a
 // non-finite sample, canaries); on BF_OK its host copy is good to read
-bf_status result_complete(bf_result* r);
+// (kernel_failed: a kernel reported an error through the result's word)
+bf_status result_complete(bf_result* r, bool* kernel_failed = nullptr);
 
 void serve_shutdown(bf_ctx* ctx);
 

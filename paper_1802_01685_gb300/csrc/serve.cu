@@ -117,6 +117,9 @@ struct ServeState {
     bool stop = false;
     bool started = false;
     cudaStream_t stream = nullptr;
+    // the status word of the loop's kernels, then the self-test's measured wait
+    int* d_err = nullptr;
+    uint64_t selftest_ns = 0;           // a wait of that limit goes before the next iteration
     // statistics
     uint64_t submitted = 0, completed = 0, cancelled = 0, rejected = 0, launches = 0;
     std::vector<double> latency_ms;
@@ -157,6 +160,7 @@ static bool admit(ServeState* S, Request* r)
     bf_result* res = nullptr;
     bf_status st = alloc_result(ctx, bank, r->opts, len, r->fs, S->stream, true, &res);
     if (st == BF_OK) {
+        res->err = S->d_err;
         st = prepare_series(ctx, r->host.data(), r->host.size(), bank->M, bank->M_pad,
                             r->opts.precision, S->stream, &r->prep, res->status);
         if (st != BF_OK) bf_result_destroy(res);
@@ -216,7 +220,7 @@ static bool admit(ServeState* S, Request* r)
             const uint32_t V = fft_lags_per_seg(bank->M, quad);
             FftSeriesBatch b{};
             b.n = 1;
-            b.err = ctx->d_err;
+            b.err = S->d_err;
             b.quad = quad ? 1 : 0;
             b.F = fft_seg_len(quad);
             b.V = V;
@@ -244,7 +248,7 @@ static bool admit(ServeState* S, Request* r)
             p.V = V;
             p.Vp = b.Vp;
             p.n_ser = 1;
-            p.err = ctx->d_err;
+            p.err = S->d_err;
             p.thr = res->thr;
             p.cand_cap = res->cand_cap;
             p.cand = res->cand;
@@ -316,6 +320,7 @@ static void scheduler(ServeState* S)
 
     for (;;) {
         std::vector<Request*> act;
+        uint64_t selftest_ns = 0;
         {
             std::unique_lock<std::mutex> lk(S->mu);
             S->cv_work.wait(lk, [&] { return S->stop || !S->queue.empty() || !S->active.empty(); });
@@ -352,7 +357,10 @@ static void scheduler(ServeState* S)
                 S->active.push_back(r);
             }
             act = S->active;
+            if (!act.empty()) std::swap(selftest_ns, S->selftest_ns);
         }
+        if (selftest_ns)
+            launch_wait_selftest(S->d_err, 0, selftest_ns, reinterpret_cast<unsigned long long*>(S->d_err + 2), S->stream);
 
         // one iteration: a chunk of template tiles of every admitted request
         NvtxRange iter_range("serve iteration");
@@ -438,7 +446,7 @@ static void scheduler(ServeState* S)
                     std::vector<Seg> one{rs.second};
                     cudaError_t e = launch_segments(ctx, one, prec, r->result->thr, r->result->cand,
                                                     r->result->cand_count, r->result->cand_cap,
-                                                    S->stream, nullptr);
+                                                    S->stream, nullptr, 0, S->d_err);
                     if (e != cudaSuccess) { r->status = cuda_fail(e, "serve launch"); r->cancel = true; }
                 } else {
                     Seg g = rs.second;
@@ -450,7 +458,7 @@ static void scheduler(ServeState* S)
             if (!shared.empty()) {
                 bf_result* r0 = shared_owner[0]->result;
                 cudaError_t e = launch_segments(ctx, shared, prec, INFINITY, r0->cand, r0->cand_count,
-                                                0, S->stream, nullptr);
+                                                0, S->stream, nullptr, 0, S->d_err);
                 if (e != cudaSuccess)
                     for (Request* r : shared_owner) { r->status = cuda_fail(e, "serve launch"); r->cancel = true; }
             }
@@ -514,10 +522,49 @@ static void scheduler(ServeState* S)
                 cudaStreamSynchronize(S->stream);
                 continue;
             }
+            // Each finished request's own words: kernel errors, non-finite samples,
+            // candidates.  A launch serves several requests and its error says not
+            // which, so on one the stream is drained and every request that is not
+            // complete fails; only then, with no result left that it concerns, is the
+            // word cleared.
+            bool failed = false, unread = false;
+            std::string why;
+            for (Request* r : done_now) {
+                if (r->cancel || r->status != BF_OK) {
+                    unread = true;
+                    continue;
+                }
+                bool kernel = false;
+                r->status = result_complete(r->result, &kernel);
+                if (r->status == BF_EINVAL)
+                    r->error = "the request's series holds a non-finite sample (NaN or infinity)";
+                else if (r->status != BF_OK)
+                    r->error = bf_last_error();
+                if (kernel) why = r->error;
+                failed = failed || kernel;
+            }
+            if (unread && !failed) {            // a request that ends without results: the word itself
+                int code = 0;
+                cudaMemcpyAsync(&code, S->d_err, sizeof code, cudaMemcpyDeviceToHost, S->stream);
+                cudaStreamSynchronize(S->stream);
+                failed = code != DEV_OK;
+                if (failed) why = "a kernel of the serving loop aborted after a timeout";
+            }
+            if (failed) {
+                cudaStreamSynchronize(S->stream);
+                cudaMemsetAsync(S->d_err, 0, sizeof(int), S->stream);
+                for (Request* r : act) {
+                    if (std::find(done_now.begin(), done_now.end(), r) != done_now.end()) continue;
+                    if (r->status == BF_OK) {
+                        r->status = BF_EDEVICE;
+                        r->error = why;
+                    }
+                    done_now.push_back(r);
+                }
+            }
             if (!done_now.empty()) {
                 std::lock_guard<std::mutex> g(S->mu);
                 const double t = now_s();
-                bf_status dev = BF_OK;
                 for (Request* r : done_now) {
                     S->active.erase(std::find(S->active.begin(), S->active.end(), r));
                     release_request_device(ctx, r);
@@ -527,15 +574,6 @@ static void scheduler(ServeState* S)
                         r->state = R_CANCELED;
                         ++S->cancelled;
                         continue;
-                    }
-                    // a kernel that gave up on a wait marks every request it served
-                    // from then on, through the context's word; then the request's
-                    // own words (non-finite samples, candidates)
-                    if (r->status == BF_OK) {
-                        r->status = dev != BF_OK ? dev : result_complete(r->result);
-                        if (r->status == BF_EDEVICE) dev = BF_EDEVICE;
-                        if (r->status == BF_EINVAL)
-                            r->error = "the request's series holds a non-finite sample (NaN or infinity)";
                     }
                     if (r->status != BF_OK) {
                         bf_result_destroy(r->result);
@@ -572,6 +610,8 @@ static bf_status ensure_started(bf_ctx* ctx)
     if (!S->started) {
         cudaSetDevice(ctx->device);
         cudaError_t e = cudaStreamCreateWithFlags(&S->stream, cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaMalloc(&S->d_err, 4 * sizeof(int));
+        if (e == cudaSuccess) e = cudaMemset(S->d_err, 0, 4 * sizeof(int));
         if (e != cudaSuccess) return cuda_fail(e, "serve stream");
         S->th = std::thread(scheduler, S);
         S->started = true;
@@ -597,6 +637,7 @@ void serve_shutdown(bf_ctx* ctx)
     }
     S->all.clear();
     if (S->stream) cudaStreamDestroy(S->stream);
+    if (S->d_err) cudaFree(S->d_err);
     delete S;
     ctx->serve = nullptr;
 }
@@ -710,6 +751,16 @@ bf_status bf_serve_cancel(bf_ctx* ctx, uint64_t ticket)
     Request* r = it->second;
     if (r->state == R_QUEUED || r->state == R_ACTIVE) r->cancel = true;
     S->cv_work.notify_all();
+    return BF_OK;
+}
+
+bf_status bf_selftest_serve(bf_ctx* ctx, uint32_t limit_us)
+{
+    if (!ctx) { set_error("NULL context"); return BF_EINVAL; }
+    if (limit_us == 0 || limit_us > 1000000u) { set_error("limit_us must be in [1, 1e6]"); return BF_EINVAL; }
+    if (!ctx->serve) { set_error("nothing has been submitted"); return BF_EINVAL; }
+    std::lock_guard<std::mutex> g(ctx->serve->mu);
+    ctx->serve->selftest_ns = (uint64_t)limit_us * 1000ull;
     return BF_OK;
 }
 
