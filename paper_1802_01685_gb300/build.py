@@ -28,7 +28,7 @@ LIB_DEBUG = os.path.join(PKG, "libbf_debug.so")
 
 SOURCES = ["api.cu", "serve.cu", "bank.cu", "prep.cu", "corr_simt.cu", "corr_tc.cu",
            "finalize.cu", "permute.cu", "noalloc.cu", "plan.cu", "predict.cu", "corr_fft.cu", "probe.cu"]
-HEADERS = ["bf_internal.h", "runtime.h", "corr_common.cuh", "synth.cuh"]
+HEADERS = ["bf_internal.h", "runtime.h", "corr_common.cuh", "device_once.h", "synth.cuh"]
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # hidden visibility: only the declarations of include/bf.h are exported

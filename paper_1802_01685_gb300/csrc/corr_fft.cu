@@ -49,6 +49,7 @@
 //    whose window holds almost none of the segment's energy are taken out of
 //    the FFT route (k_fft_flags) and computed directly (k_fft_fixup).
 #include "corr_common.cuh"
+#include "device_once.h"
 #include "synth.cuh"
 #include "runtime.h"
 
@@ -1502,35 +1503,30 @@ __global__ void __launch_bounds__(FIX_T) k_fft_fixup(const __grid_constant__ Fft
     }
 }
 
+template <typename K>
+cudaError_t smem_opt_in(K kernel, size_t bytes)
+{
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
 cudaError_t fft_attributes()
 {
-    static bool done = false;
-    if (done) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(k_corr_fft<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CORR_SMEM);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_corr_fft<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CORR_SMEM);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_corr_fft<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CORR_SMEM);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_corr_fft<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CORR_SMEM);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_fft_series<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FFT_SMEM);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_fft_series<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FFT_SMEM);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_fft_bank_real, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BANK_SMEM);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_fft_bank_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FFT_SMEM);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_welch_segments, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FFT_SMEM);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_template_power_dot, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FFT_SMEM);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_fft_fixup<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FIX_SMEM);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_fft_fixup<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FIX_SMEM);
-    if (e == cudaSuccess) done = true;
-    return e;
+    static DeviceOnce once;
+    return once.run([] {
+        cudaError_t e = smem_opt_in(k_corr_fft<false, false>, CORR_SMEM);
+        if (e == cudaSuccess) e = smem_opt_in(k_corr_fft<false, true>, CORR_SMEM);
+        if (e == cudaSuccess) e = smem_opt_in(k_corr_fft<true, false>, CORR_SMEM);
+        if (e == cudaSuccess) e = smem_opt_in(k_corr_fft<true, true>, CORR_SMEM);
+        if (e == cudaSuccess) e = smem_opt_in(k_fft_series<true>, FFT_SMEM);
+        if (e == cudaSuccess) e = smem_opt_in(k_fft_series<false>, FFT_SMEM);
+        if (e == cudaSuccess) e = smem_opt_in(k_fft_bank_real, BANK_SMEM);
+        if (e == cudaSuccess) e = smem_opt_in(k_fft_bank_pair, FFT_SMEM);
+        if (e == cudaSuccess) e = smem_opt_in(k_welch_segments, FFT_SMEM);
+        if (e == cudaSuccess) e = smem_opt_in(k_template_power_dot, FFT_SMEM);
+        if (e == cudaSuccess) e = smem_opt_in(k_fft_fixup<false>, FIX_SMEM);
+        if (e == cudaSuccess) e = smem_opt_in(k_fft_fixup<true>, FIX_SMEM);
+        return e;
+    });
 }
 
 }  // namespace

@@ -33,6 +33,7 @@
 // error code in the status word, drains its own copies and MMAs, frees TMEM
 // and returns.
 #include "corr_common.cuh"
+#include "device_once.h"
 
 namespace bfi {
 
@@ -692,21 +693,20 @@ static cudaError_t set_attr()
                                 (int)Geo<LT>::SMEM);
 }
 
-static bool g_attr_done = false;
-
 cudaError_t corr_tc_set_attributes()
 {
-    if (g_attr_done) return cudaSuccess;
-    cudaError_t e = set_attr<1, 512>();
-    if (e == cudaSuccess) e = set_attr<1, 256>();
-    if (e == cudaSuccess) e = set_attr<3, 256>();
-    if (e == cudaSuccess) e = set_attr<1, 128>();
-    if (e == cudaSuccess) e = set_attr<3, 128>();
-    if (e == cudaSuccess) g_attr_done = true;
-    return e;
+    static DeviceOnce once;
+    return once.run([] {
+        cudaError_t e = set_attr<1, 512>();
+        if (e == cudaSuccess) e = set_attr<1, 256>();
+        if (e == cudaSuccess) e = set_attr<3, 256>();
+        if (e == cudaSuccess) e = set_attr<1, 128>();
+        if (e == cudaSuccess) e = set_attr<3, 128>();
+        return e;
+    });
 }
 
-// Self-test of the bounded wait above: one mbarrier expecting one arrival,
+// Self-test of the bounded wait (mbar_wait): one mbarrier expecting one arrival,
 // which thread 0 of warp 1 makes only when `signal` is set, and warp 0 waiting
 // on it with the given limit.  A timeout is recorded in the status word as in
 // the correlation kernel; waited[0] gets the nanoseconds spent waiting.
