@@ -324,7 +324,11 @@ typedef struct {
     int32_t candidates_overflow;   /* 1 if more than max_candidates: map partial */
     float threshold;               /* kappa / sqrt(M)                           */
     uint32_t hist_bins;
-    double kernel_ms;              /* correlation kernel time (synchronous calls) */
+    double kernel_ms;              /* time of the correlation kernels, with a
+                                      generated bank's synthesis and the FFT
+                                      route's segment spectra (synchronous
+                                      calls); of a plan's run without its
+                                      copies, preparation included          */
     int32_t tile_lags;             /* lags per tile of the kernel that ran      */
 } bf_result_info;
 

@@ -912,13 +912,16 @@ int gen_autotune(bf_ctx* ctx, const bf_bank* bank, const bf_opts& o, const std::
     return choose_lag_tile(ctx, gen_chunk_segments(bank, o, segs, g, 0, 0)[0], o.precision, strm);
 }
 
-// forks the synthesis stream from strm and makes chunk 0; gen_launch joins it
-cudaError_t gen_begin(bf_ctx* ctx, const bf_bank* bank, const bf_opts& o, cudaStream_t strm, GenRing& g)
+// forks the synthesis stream from strm and makes chunk 0 (timed: between the
+// context's events 2 and 3); gen_launch joins it
+cudaError_t gen_begin(bf_ctx* ctx, const bf_bank* bank, const bf_opts& o, cudaStream_t strm, GenRing& g, bool timed)
 {
     // the synthesis stream starts after everything already queued on the main one
     cudaError_t e = cudaEventRecord(g.ev.start, strm);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->aux, g.ev.start, 0);
+    if (e == cudaSuccess && timed) e = cudaEventRecord(ctx->ev[2], ctx->aux);
     if (e == cudaSuccess) e = gen_synth(bank, o, g, 0, 0, ctx->aux);
+    if (e == cudaSuccess && timed) e = cudaEventRecord(ctx->ev[3], ctx->aux);
     if (e == cudaSuccess) e = cudaEventRecord(g.ev.made[0], ctx->aux);
     return e;
 }
@@ -1551,7 +1554,7 @@ bf_status bf_correlate(bf_ctx* ctx, const bf_bank* bank, const float* const* ser
         st = gen_prepare(ctx, bank, o, r, &ring);
         if (st) return st;
         join.aux = ctx->aux;
-        const cudaError_t eg = gen_begin(ctx, bank, o, strm, ring);
+        const cudaError_t eg = gen_begin(ctx, bank, o, strm, ring, sync);
         if (eg != cudaSuccess) return cuda_fail(eg, "template synthesis");
     }
 
@@ -1633,6 +1636,13 @@ bf_status bf_correlate(bf_ctx* ctx, const bf_bank* bank, const float* const* ser
         e = cudaStreamSynchronize(strm);
         float ms = 0.f;
         cudaEventElapsedTime(&ms, ctx->ev[0], ctx->ev[1]);
+        if (!fft && bank->generated) {
+            // the first chunk's synthesis, as far as it ran ahead of that
+            float made = 0.f, ahead = 0.f;
+            cudaEventElapsedTime(&made, ctx->ev[2], ctx->ev[3]);
+            cudaEventElapsedTime(&ahead, ctx->ev[2], ctx->ev[0]);
+            ms += std::max(0.f, std::min(made, ahead));
+        }
         r->kernel_ms = ms;
         if (e != cudaSuccess) return cuda_fail(e, "correlation");
         st = result_complete(r);

@@ -459,7 +459,9 @@ struct bf_ctx {
     cudaStream_t aux = nullptr;         // template synthesis of generated banks
     std::unique_ptr<bfi::Allocator> mem;
     std::unique_ptr<bfi::HostPool> host_mem;
-    cudaEvent_t ev[2] = {nullptr, nullptr};   // kernel time of synchronous calls (under launch_mu)
+    // kernel time of synchronous calls (under launch_mu): the correlation's begin
+    // and end, the begin and end of the first chunk's synthesis beside it
+    cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
     int* d_err = nullptr;               // kernel status word
     std::mutex launch_mu;               // serialises use of d_err / stream
     bfi::ServeState* serve = nullptr;   // owned; freed by serve_shutdown

@@ -137,7 +137,8 @@ void gen_point_segment(Seg& g, int precision, size_t k0, const void* slot0, cons
 cudaError_t fft_template_spectra(const bf_bank* bank, size_t row0, size_t nrows, float* scratch,
                                  size_t scratch_rows, const float2* tw, float2* out, int n_sm, cudaStream_t st);
 bf_status gen_prepare(bf_ctx* ctx, const bf_bank* bank, const bf_opts& o, bf_result* r, GenRing* g);
-cudaError_t gen_begin(bf_ctx* ctx, const bf_bank* bank, const bf_opts& o, cudaStream_t strm, GenRing& g);
+cudaError_t gen_begin(bf_ctx* ctx, const bf_bank* bank, const bf_opts& o, cudaStream_t strm, GenRing& g,
+                      bool timed = false);
 cudaError_t gen_launch(bf_ctx* ctx, const bf_bank* bank, const bf_opts& o, const std::vector<Seg>& segs,
                        bf_result* r, cudaStream_t strm, int lt, GenRing& g);
 // the tile shape for a generated bank: the first chunk synthesised (on strm,
