@@ -384,8 +384,9 @@ void build_segments(const std::vector<PreparedSeries*>& ser, const std::vector<u
 }
 
 // Times both tile shapes of the tensor-core kernel on a zero series (its cost
-// does not depend on the data) against up to 4 of the segment's template
-// tiles, two waves of tiles each, and keeps the faster one per context.
+// does not depend on the data) against 1, 2 or 4 of the segment's template
+// tiles, whole rounds of one tile per SM (two of the larger shape, four of the
+// smaller), as most of a long search is, and keeps the faster one per context.
 int choose_lag_tile(bf_ctx* ctx, const Seg& g, int precision, cudaStream_t st)
 {
     if (precision != BF_BF16) return TC_TILE_L / 2;      // the split routes have one shape
@@ -395,8 +396,8 @@ int choose_lag_tile(bf_ctx* ctx, const Seg& g, int precision, cudaStream_t st)
         auto it = ctx->tuned.find(key);
         if (it != ctx->tuned.end()) return it->second;
     }
-    const uint32_t ntt = std::min<uint32_t>(g.n_tt, 4);
-    const uint64_t L = (uint64_t)ctx->n_sm * TC_TILE_L * 2 / ntt + 1;
+    const uint32_t ntt = g.n_tt >= 4 && ctx->n_sm % 2 == 0 ? 4 : g.n_tt >= 2 ? 2 : 1;
+    const uint64_t L = (uint64_t)ctx->n_sm * 2 / ntt * TC_TILE_L;
     const uint64_t rows = ceil_div(L, TC_TILE_L) * TC_TILE_L + g.M_pad + 64;
     Allocator& mem = *ctx->mem;
     void* yh = mem.alloc(rows * 16);

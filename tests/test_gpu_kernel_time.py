@@ -1,5 +1,6 @@
-"""What the times that a result reports cover: a generated bank's kernel_ms
-includes the synthesis of its templates, whenever it ran."""
+"""What times cover: a generated bank's kernel_ms includes the synthesis of its
+templates, whenever it ran; the autotuner's probe of the 256-lag tile runs whole
+tiles only, as long searches do."""
 import numpy as np
 import pytest
 
@@ -37,3 +38,25 @@ def test_kernel_time_covers_the_synthesis(ctx):
     assert ms(gen) >= ms(stored) + 0.05
     bf.bf_bank_destroy(stored)
     bf.bf_bank_destroy(gen)
+
+
+def test_autotuner_times_whole_tiles():
+    """A fresh context's first BF16 search runs the probe: four launches of each
+    shape and no second launch of halves."""
+    ctx = bf.bf_init()
+    try:
+        fs, T = 2048.0, 1.0
+        spec = synth.grid_spec([synth.LINEAR], [synth.ASC], [T], 50.0, 900.0, 24, 16)     # 384: three template tiles
+        bank = bf.bf_bank_create_grid(ctx, spec, fs, T, bf.BF_BANK_SPLIT_BF16)
+        x = np.random.default_rng(2).standard_normal(20000).astype(np.float32)
+
+        def launches():
+            n0 = bf.bf_kernel_launches()
+            bf.bf_result_destroy(bf.bf_correlate(ctx, bank, [x], fs, bf.make_opts(precision="bf16")))
+            return bf.bf_kernel_launches() - n0
+
+        first, second = launches(), launches()
+        assert first - second == 8, (first, second)
+        bf.bf_bank_destroy(bank)
+    finally:
+        bf.bf_destroy(ctx)
