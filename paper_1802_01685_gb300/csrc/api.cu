@@ -735,7 +735,7 @@ cudaError_t clear_result(bf_result* r, cudaStream_t st)
     add(r->cand_count, 2 * sizeof(unsigned int));
     if (r->hist) add(r->hist, S * r->nbins * 4);
     if (r->map) add(r->map, r->map_total * 4);
-    return launch_clear(p, st);
+    return launch_clear(p, r->ctx->n_sm, st);
 }
 
 // Finalize kernels for a result whose correlation launches are enqueued.

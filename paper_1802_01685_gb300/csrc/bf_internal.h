@@ -346,7 +346,7 @@ struct ClearParams {
     uint32_t* ptr[5];
     uint64_t words[5];
 };
-cudaError_t launch_clear(const ClearParams& p, cudaStream_t s);
+cudaError_t launch_clear(const ClearParams& p, int n_sm, cudaStream_t s);
 
 constexpr int MAX_FIN = 128;        // series per finalize / paint launch
 struct FinalizeParams {

@@ -31,11 +31,11 @@ __global__ void __launch_bounds__(256) k_clear(const __grid_constant__ ClearPara
     }
 }
 
-cudaError_t launch_clear(const ClearParams& p, cudaStream_t s)
+cudaError_t launch_clear(const ClearParams& p, int n_sm, cudaStream_t s)
 {
     uint64_t most = 0;
     for (int r = 0; r < p.n; ++r) most = std::max(most, p.words[r] / 4);
-    const unsigned blocks = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((most + 255) / 256, 152 * 8));
+    const unsigned blocks = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((most + 255) / 256, (uint64_t)n_sm * 8));
     count_launches(1);
     k_clear<<<blocks, 256, 0, s>>>(p);
     return cudaGetLastError();
