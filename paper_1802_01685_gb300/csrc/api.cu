@@ -789,7 +789,7 @@ bf_status finalize_result(bf_ctx* ctx, const bf_bank* bank, bf_result* r, cudaSt
                 p.n_hist = (uint64_t)S * r->nbins;
             }
         }
-        e = launch_publish(p, st);
+        e = launch_publish(p, ctx->n_sm, st);
     }
     if (e != cudaSuccess) return cuda_fail(e, "finalize");
     return BF_OK;

@@ -391,7 +391,7 @@ cudaError_t launch_coincidence(const float* A, const float* B, uint32_t nt, uint
                                uint32_t dt, unsigned int* out, int n_sm, cudaStream_t s);
 cudaError_t launch_skewnorm_fit(const float* v, uint64_t n, double* acc, double* out, int n_sm,
                                 cudaStream_t s);
-cudaError_t launch_publish(const PublishParams& p, cudaStream_t s);
+cudaError_t launch_publish(const PublishParams& p, int n_sm, cudaStream_t s);
 cudaError_t launch_paint(const Candidate* cand, const unsigned int* count,
                          unsigned int cap, const ChirpDev* params,
                          const FinalizeParams& p, uint32_t M, double fs, double dt,

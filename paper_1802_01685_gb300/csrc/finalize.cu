@@ -98,10 +98,12 @@ cudaError_t launch_finalize(const FinalizeParams& p, uint32_t K, uint32_t nbins,
     return cudaGetLastError();
 }
 
-cudaError_t launch_publish(const PublishParams& p, cudaStream_t s)
+// The grid is for the templates or the histograms' words, whichever are more.
+cudaError_t launch_publish(const PublishParams& p, int n_sm, cudaStream_t s)
 {
-    const unsigned b = (p.K + 255) / 256;
-    if (b == 0) return cudaSuccess;
+    if (p.K == 0) return cudaSuccess;
+    const uint64_t work = std::max<uint64_t>(p.K, p.hist ? p.n_hist : 0);
+    const unsigned b = (unsigned)std::min<uint64_t>((work + 255) / 256, std::max<uint64_t>((p.K + 255) / 256, (uint64_t)n_sm * 8));
     count_launches(1);
     k_publish<<<b, 256, 0, s>>>(p);
     return cudaGetLastError();

@@ -1,6 +1,8 @@
 """What times cover: a generated bank's kernel_ms includes the synthesis of its
 templates, whenever it ran; the autotuner's probe of the 256-lag tile runs whole
-tiles only, as long searches do."""
+tiles only, as long searches do; a histogram of many bins does not rule a call."""
+import time
+
 import numpy as np
 import pytest
 
@@ -60,3 +62,28 @@ def test_autotuner_times_whole_tiles():
         bf.bf_bank_destroy(bank)
     finally:
         bf.bf_destroy(ctx)
+
+
+def test_many_bins_for_few_templates(ctx):
+    """The last kernel copies the histograms to host memory.  A million bins of 64
+    templates are 4 MB, which the whole GPU writes in 20 us of an 80 us call; by
+    the one block that 64 templates need they took 800."""
+    fs = 2048.0
+    spec = synth.grid_spec([synth.LINEAR], [synth.ASC], [1.0], 60.0, 480.0, 8, 8)
+    bank = bf.bf_bank_create_grid(ctx, spec, fs, 1.0, bf.BF_BANK_SPLIT_BF16)
+    x = np.random.default_rng(6).standard_normal(8192).astype(np.float32)
+
+    def call(bins):
+        best = 1e9
+        for _ in range(12):
+            t0 = time.perf_counter()
+            res = bf.bf_correlate(ctx, bank, [x], fs, bf.make_opts(hist_bins=bins))
+            best = min(best, time.perf_counter() - t0)
+            out = bf.bf_result_copy_to_host(res, 0)
+            bf.bf_result_destroy(res)
+        want = np.bincount(np.minimum((out["max"] * np.float32(bins)).astype(np.int64), bins - 1), minlength=bins)
+        np.testing.assert_array_equal(out["hist"], want)
+        return best
+
+    assert call(1_000_000) < 4.0 * call(1024)
+    bf.bf_bank_destroy(bank)
