@@ -503,7 +503,7 @@ void bf_result_destroy(bf_result* r);
  * made on the context's second stream) is captured in the graph too.  Runs
  * of one plan must
  * not overlap on the GPU, nor a run with asynchronous copies of the previous
- * run's result.
+ * run's result.  bf_plan_destroy waits for the last run.
  */
 typedef struct bf_plan bf_plan;
 bf_status bf_plan_create(bf_ctx* ctx, const bf_bank* bank, const size_t* lengths,

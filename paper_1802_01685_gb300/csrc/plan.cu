@@ -1,8 +1,9 @@
 // Search plans: one search shape captured once as a CUDA graph and replayed.
 // Every buffer of the search (result, prepared series, scratch) is allocated
 // at creation; a run copies the new series in and launches the graph, so a
-// repeated search costs one graph launch instead of one launch per kernel and
-// memset (six or more per series plus the correlation and finalize kernels).
+// repeated search costs one graph launch instead of one launch per kernel (one to
+// clear the outputs, four to prepare up to 64 series, the correlation's, and two
+// or more to finish).
 #include <cmath>
 #include <cstring>
 
@@ -19,6 +20,7 @@ struct bf_plan {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     uint64_t launches_per_run = 0;      // kernel nodes in the graph
+    cudaEvent_t last = nullptr;         // the last run on a caller's stream
 };
 
 using namespace bfi;
@@ -31,6 +33,12 @@ void bf_plan_destroy(bf_plan* p)
     if (p->ctx) {
         cudaSetDevice(p->ctx->device);
         cudaStreamSynchronize(p->ctx->stream);
+        // a run writes the buffers that go back below for other results, page-locked
+        // host memory among them
+        if (p->last) {
+            cudaEventSynchronize(p->last);
+            cudaEventDestroy(p->last);
+        }
     }
     if (p->exec) cudaGraphExecDestroy(p->exec);
     if (p->graph) cudaGraphDestroy(p->graph);
@@ -166,6 +174,8 @@ bf_status bf_plan_create(bf_ctx* ctx, const bf_bank* bank, const size_t* lengths
                                  : (fst != BF_OK ? fst : cuda_fail(e, "cudaStreamEndCapture"));
     }
     p->graph = graph;
+    e = cudaEventCreateWithFlags(&p->last, cudaEventDisableTiming);
+    if (e != cudaSuccess) return cuda_fail(e, "plan events");
     p->launches_per_run = g_launches.load() - l0;
     g_launches.fetch_sub(p->launches_per_run);      // counted when the graph runs
     e = cudaGraphInstantiate(&p->exec, graph, 0);
@@ -196,6 +206,7 @@ bf_status bf_plan_run(bf_plan* p, const float* const* series, void* stream, cons
     if (e == cudaSuccess) e = cudaGraphLaunch(p->exec, strm);
     if (e == cudaSuccess) count_launches(p->launches_per_run);
     if (sync) cudaEventRecord(ctx->ev[1], strm);
+    else if (e == cudaSuccess) e = cudaEventRecord(p->last, strm);
     if (e == cudaSuccess && sync) e = cudaStreamSynchronize(strm);
     if (sync) {
         float ms = 0.f;
