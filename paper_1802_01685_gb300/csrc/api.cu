@@ -599,8 +599,10 @@ bf_status resolve_opts(const bf_bank* bank, const bf_opts* in, bf_opts* o)
     return BF_OK;
 }
 
-// Largest host copy of a result: a search of 65,536 templates in four series
-// (3.2 MB).  Larger ones are copied when asked for, at the link's full rate.
+// Largest host copy of a result.  It bounds page-locked memory, sixteen such results
+// filling the context's pool, and takes in a search of 65,536 templates in four
+// series (3.2 MB); writing 4 MB takes 20 us of a call (79.8 -> 100.6 us).  Larger
+// results are copied when asked for.
 constexpr size_t HOST_COPY_BYTES = size_t(4) << 20;
 
 // Allocates and zeroes the outputs of a result for series of the given lengths.

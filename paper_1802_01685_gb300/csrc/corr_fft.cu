@@ -128,8 +128,9 @@ __global__ void k_fft_tables(float2* __restrict__ tw)
     }
 }
 
-// Work array z (complex, index i stored at i + i/16), twiddle tables, and, in
-// the correlation kernels, a second work array z2 and the staged spectrum x.
+// Work array z (complex, index i stored at i + i/16), twiddle tables, and, for the
+// template spectra of the real route (TWO), a second work array z2 and the staged
+// row x.
 struct Smem {
     float2* z;
     const float2* tw;
@@ -137,11 +138,11 @@ struct Smem {
     float2* x;
 };
 
-template <bool CORR>
+template <bool TWO>
 __device__ __forceinline__ Smem smem_setup(const float2* __restrict__ tw_global)
 {
     extern __shared__ __align__(16) float2 fsm[];
-    Smem m{fsm, fsm + ZPAD, CORR ? fsm + ZPAD + TW_N : nullptr, CORR ? fsm + 2 * ZPAD + TW_N : nullptr};
+    Smem m{fsm, fsm + ZPAD, TWO ? fsm + ZPAD + TW_N : nullptr, TWO ? fsm + 2 * ZPAD + TW_N : nullptr};
     float4* dst = reinterpret_cast<float4*>(fsm + ZPAD);
     const float4* src = reinterpret_cast<const float4*>(tw_global);
     for (int i = threadIdx.x; i < TW_N / 2; i += blockDim.x) dst[i] = __ldg(src + i);
@@ -254,10 +255,8 @@ __device__ __forceinline__ void dft16(float (&r)[16], float (&i)[16])
 // takes the 16-point DFT and writes out[(j / NS) 16 NS + j mod NS + q NS].
 // Padded addresses (i + i/16) are a per-thread base plus constant offsets.
 // The second half of a pass, from the 16 inputs already in registers, into
-// the work array dst; it ends with a barrier, before which the calling
-// thread's pending cp.async groups but WAIT_CP are waited for (WAIT_CP < 0:
-// no wait).
-template <int SIGN, int NS, int WAIT_CP = -1>
+// the work array dst; it ends with a barrier.
+template <int SIGN, int NS>
 __device__ __forceinline__ void pass16_from(const Smem& m, float2* dst, float (&vr)[16], float (&vi)[16])
 {
     const int j = threadIdx.x;
@@ -297,13 +296,12 @@ __device__ __forceinline__ void pass16_from(const Smem& m, float2* dst, float (&
         const int off = NS == 1 ? q : NS == 16 ? 17 * q : 272 * q;
         dst[wb + off] = make_float2(vr[p], vi[p]);
     }
-    if (WAIT_CP >= 0) cp_async_wait<(WAIT_CP >= 0 ? WAIT_CP : 0)>();
     __syncthreads();
 }
 
 // A pass from work array src to dst; in place (src == dst) every thread's
 // reads complete at a barrier before the first write.
-template <int SIGN, int NS, int WAIT_CP = -1, bool IN_PLACE = true>
+template <int SIGN, int NS, bool IN_PLACE = true>
 __device__ __forceinline__ void pass16(const Smem& m, const float2* src, float2* dst)
 {
     const int j = threadIdx.x;
@@ -316,7 +314,7 @@ __device__ __forceinline__ void pass16(const Smem& m, const float2* src, float2*
         vi[r] = v.y;
     }
     if (IN_PLACE) __syncthreads();
-    pass16_from<SIGN, NS, WAIT_CP>(m, dst, vr, vi);
+    pass16_from<SIGN, NS>(m, dst, vr, vi);
 }
 
 template <int SIGN>
@@ -593,8 +591,8 @@ __global__ void __launch_bounds__(FT, 1) k_fft_bank_real(const float* __restrict
         const uint32_t qn = q + gridDim.x;
         if (qn < n_rows) stage(qn);
         cp_async_commit();
-        pass16<-1, 16, -1, false>(m, m.z, m.z2);
-        pass16<-1, 256, -1, false>(m, m.z2, m.z);
+        pass16<-1, 16, false>(m, m.z, m.z2);
+        pass16<-1, 256, false>(m, m.z2, m.z);
         real_spectrum_quads(m, base_f, base_r, spec + (size_t)q * FN);
         if (qn >= n_rows) break;
         q = qn;
