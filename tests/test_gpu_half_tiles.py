@@ -36,13 +36,21 @@ def test_halves_equal_whole_tiles(ctx, prec, quad):
     rng = np.random.default_rng(3)
     lags = [1, 127, 128, 129, 255, 256, 257, 385, 700]
     xs = [rng.standard_normal(M - 1 + n).astype(np.float32) for n in lags]
-    fill = rng.standard_normal(60000).astype(np.float32)
-    opts = bf.make_opts(precision=prec, want_tails=True, kappa=3.0)
+    # the batch's first tiles are the short series', in whole rounds of one tile per
+    # SM; alone each has at most 9, in halves
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    fill = rng.standard_normal(M - 1 + 2 * n_sm * 256).astype(np.float32)
+    tt = -(-(2 if quad else 1) * 160 // 128)                  # template tiles
+    tiles = [-(-n // 256) * tt for n in lags]
+    assert 2 * max(tiles) <= n_sm and (sum(tiles) + 2 * n_sm * tt) // n_sm * n_sm >= sum(tiles)
+    opts = bf.make_opts(precision=prec, want_tails=True, kappa=3.0, tile_lags=256)
     try:
-        batch = bf.bf_correlate(ctx, bank, xs + [fill], FS, opts)          # 228 fill tiles a template tile
+        batch = bf.bf_correlate(ctx, bank, xs + [fill], FS, opts)
+        assert bf.bf_result_info_get(batch).tile_lags == 256
         tails = bf.bf_result_copy_tails(batch)
         for s, x in enumerate(xs):
             alone = bf.bf_correlate(ctx, bank, [x], FS, opts)
+            assert bf.bf_result_info_get(alone).tile_lags == 256
             a, b = bf.bf_result_copy_to_host(alone, 0), bf.bf_result_copy_to_host(batch, s)
             np.testing.assert_array_equal(a["max"], b["max"], err_msg=f"{lags[s]} lags")
             np.testing.assert_array_equal(a["argmax"], b["argmax"], err_msg=f"{lags[s]} lags")
