@@ -1,6 +1,6 @@
 """What the FFT route's epilogue reduces: a NaN of an overflowing transform
-reaches the maximum, and the sum of rho^2 leaves FP32 after a thread's own 32
-terms, lanes and segments being added in FP64."""
+reaches the maximum, and the sum of rho^2 rounds in FP32 over chains of 32 terms
+only, those being added as pairs of FP32 values and then in FP64."""
 import numpy as np
 import pytest
 
