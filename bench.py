@@ -48,7 +48,7 @@ UNIT = "correlations/s"
 # Keyed by (hash of the kernel source the counters were taken on, lags per
 # tile); a changed kernel reports null until it is captured again.
 TRAFFIC_BYTES_PER_TEMPLATE_TILE = {
-    ("176b52ad1019a23f", 256): (272.54e6 + 0.59e6) / 128,   # the 16 s x 16,384-template capture
+    ("fd95644241c321f8", 256): (272.21e6 + 0.54e6) / 128,   # the 16 s x 16,384-template capture
 }
 
 
@@ -564,8 +564,8 @@ def run_fft(ctx, bf, w, xs, ctrl, corr_per_step, alu, steps=3):
                          "frac": round(fft_flops / (k_ms / 1e3) / 1e12 / alu["fp32_tflops"], 4),
                          "peak_source": "measured FP32 FMA rate (alu_peaks)",
                          "work": "5 N log2 N nominal flops per N-point complex transform",
-                         "note": "on-chip bound: the profile puts the L1 data pipe at 62 %, the FP32 "
-                                 "pipe at 56 % and issue at 54 % of their peaks; no DRAM bound"},
+                         "note": "on-chip bound: the profile puts the L1 data pipe at 63 %, the FP32 "
+                                 "pipe at 57 % and issue at 55 % of their peaks; no DRAM bound"},
             "roofline_smem": smem_roofline(n_transforms, k_ms, clocks),
             "clocks": clocks,
             "note": "FP32 complex FFTs of 8192 points carrying real segments of 16384 samples "
@@ -579,9 +579,9 @@ def run_fft(ctx, bf, w, xs, ctrl, corr_per_step, alu, steps=3):
 # shared-memory wavefronts per 8192-point transform of the real-route
 # correlation kernel (ncu l1tex__data_pipe_lsu_wavefronts_mem_shared.sum over
 # the transforms of the 16 s x 16,384-template case): the passes' loads and
-# stores, the template's records and the twiddles (the segment spectrum, the
-# norms and the mirrors' shuffles cross the same pipe, another 980)
-FFT_SMEM_WAVEFRONTS = 3600
+# stores, the template's records, the twiddles and the threads' sums (the segment
+# spectrum, the norms and the mirrors' shuffles cross the same pipe, another 970)
+FFT_SMEM_WAVEFRONTS = 3630
 
 
 def torch_device_index() -> int:

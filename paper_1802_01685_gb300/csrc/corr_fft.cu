@@ -920,16 +920,16 @@ __device__ __forceinline__ float2 root64(int a)
 // are hardware barriers.
 //
 // What bounds it: the L1 data pipe, 4.6 K wavefronts a transform at five
-// segments a template (work array 2.2 K, spectra 1.5 K, norms, mirrors and
-// twiddles 0.9 K), beside 4.1 K cycles of FP32 and 4.0 K of issue (62, 56 and
-// 54 % busy).  A transform takes 7.4 K cycles (6.3 K at 84 segments a template):
+// segments a template (work array 2.2 K, spectra 1.5 K, norms, mirrors, twiddles
+// and sums 0.9 K), beside 4.2 K cycles of FP32 and 4.1 K of issue (63, 57 and
+// 55 % busy).  A transform takes 7.3 K cycles (6.2 K at 84 segments a template):
 // four warps a scheduler do not overlap the three any further, and the registers
 // and the shared memory hold no third group.  16 s x 16,384 templates of 4096
-// samples (81,920 transforms) run 1.91 ms; the form it replaced (one CTA-wide
+// samples (81,920 transforms) run 1.90 ms; the form it replaced (one CTA-wide
 // group with the template in registers, unpacked arithmetic, the radix-2 stage
 // last through shared memory, 9 K warp instructions more per transform and four
 // CTA-wide barriers) ran 2.60.  The 64 s x 4 series x 65,536 template step went
-// from 163.7 to 113.4 ms.  Unpacked twiddle products (rotate1) are 1 % of that.
+// from 163.7 to 112.0 ms.  Unpacked twiddle products (rotate1) are 1 % of that.
 template <bool QUAD, bool DENSE>
 __global__ void __launch_bounds__(FT, 1) k_corr_fft(const __grid_constant__ FftParams p, uint32_t total)
 {
