@@ -303,6 +303,9 @@ void bf_opts_default(bf_opts* opts);
  * returns BF_EINVAL with no result; after a call on a stream, or a plan run
  * on a stream, bf_result_check reads it once the stream has synchronised; a
  * served request fails with BF_EINVAL.
+ * Finite samples so large that a transform of BF_FFT_FP32 overflows FP32
+ * (above about 1e33) give NaN maxima and sigmas for their series; a
+ * quadrature bank's outputs, which are squared, are infinite from about 1e15.
  * BF_EINVAL on a bad length, rate, range, a precision whose layout the bank
  * lacks, or a non-finite sample; BF_EDEVICE if a kernel reported an internal
  * timeout.
